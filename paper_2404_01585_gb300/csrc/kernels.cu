@@ -1012,12 +1012,17 @@ static void ws_free(Workspace &w) {
 // Capacity is kept in patterns and in window slots (patterns x Wmax) separately, so a large
 // batch with small windows followed by a small batch with large windows never allocates the
 // product of the two.
-static int ws_ensure(const DeviceGraph *g, Workspace &w, int32_t P, int32_t Wmax, int32_t sel) {
+static int ws_ensure(DeviceGraph *g, Workspace &w, int32_t P, int32_t Wmax, int32_t sel) {
     const int64_t slots = (int64_t)P * Wmax;
     if (P <= w.P && slots <= w.slots && (int64_t)P * sel <= w.sel_slots && w.h_ctl) return FLEXIS_OK;
     const int32_t nP = std::max(P, w.P);
     const int64_t nSlots = std::max(slots, w.slots);
     const int64_t nSel = std::max((int64_t)P * sel, w.sel_slots);
+    // the captured round loop holds the old buffers' addresses: it goes with them
+    if (&w == &g->ws && g->round_exec) {
+        cudaGraphExecDestroy(g->round_exec);
+        g->round_exec = nullptr;
+    }
     ws_free(w);
     const size_t words = (size_t)g->view.words;
     int64_t b = 0;
@@ -1026,7 +1031,6 @@ static int ws_ensure(const DeviceGraph *g, Workspace &w, int32_t P, int32_t Wmax
         return cudaMalloc(ptr, std::max<size_t>(bytes, 16));
     };
     CK(alloc((void **)&w.st, sizeof(PatState) * nP));
-    CK(cudaMemset(w.st, 0, sizeof(PatState) * nP));
     CK(alloc((void **)&w.used, sizeof(uint32_t) * words * nP));
     CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nP));
     w.clean = 0;
