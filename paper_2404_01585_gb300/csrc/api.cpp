@@ -105,6 +105,11 @@ EvalConfig config_for(const flexis_graph *g, int32_t P) {
     int wmin = std::max(16, std::min(wmax, 16384 / std::max(1, P)));
     if (g->opt.window_max > 0) wmax = g->opt.window_max;
     if (g->opt.window_min > 0) wmin = g->opt.window_min;
+    // the streaming greedy, unless the caller sets up the windowed rounds himself (or a label may
+    // have more roots than it can number)
+    const flexis_options &o = g->opt;
+    c.streamed = o.window_max <= 0 && o.window_min <= 0 && o.search_budget == 0 && o.split_pieces == 0 &&
+                 o.sub_searches <= 0 && g->hg.nv < (int64_t)60'000'000;
     c.w_min = std::min(wmin, wmax);
     c.w_max = wmax;
     c.search_blocks = g->opt.search_blocks;
@@ -124,8 +129,10 @@ constexpr int32_t EXACT_MIS_DEFAULT_INSTANCES = 2048, EXACT_MIS_MAX_INSTANCES = 
 constexpr int32_t EXACT_MIS_BATCH = 64;  // patterns whose maps are materialised at once
 
 void enum_config(const flexis_graph *g, const Plan *plans, int64_t n, EvalConfig &c) {
-    c.count_maps = c.exact_mis = false;
+    c.count_maps = c.exact_mis = c.want_mni = c.cyclic = false;
     for (int64_t i = 0; i < n; i++) {
+        c.want_mni |= plans[i].want_mni != 0;
+        c.cyclic |= plans[i].status == FLEXIS_OK && plans[i].n_edges >= plans[i].n;
         c.count_maps |= plans[i].count_maps != 0;
         c.exact_mis |= plans[i].exact_mis != 0;
     }
@@ -207,7 +214,7 @@ int eval_plans(flexis_graph *g, std::vector<Plan> &plans, flexis_support_result 
     EvalConfig cfg = config_for(g, (int32_t)std::min<int64_t>(P, INT32_MAX));
     enum_config(g, plans.data(), P, cfg);
     int64_t per = 1, fr = 0;
-    dev_pattern_bytes(g->dg, cfg.w_max, cfg.record_selected, &per);
+    dev_pattern_bytes(g->dg, cfg.w_max, cfg.record_selected, cfg.streamed, &per);
     dev_free_bytes(g->dg, &fr);
     const int64_t budget = std::max<int64_t>(fr / 3, 256ll << 20);
     int64_t chunk = std::max<int64_t>(1, std::min<int64_t>({P, budget / std::max<int64_t>(per, 1), 1 << 22}));

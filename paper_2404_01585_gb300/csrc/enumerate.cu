@@ -158,11 +158,12 @@ __global__ void __launch_bounds__(ENUM_THREADS) k_extend(EnumPass E) {
             bytes += 32;
             ok = vertex_fits(E.G, W.t[0], W.L.deg[0], W.need[W.L.vert[0]]);
         }
-        if (ok) ok = enter_level(E.G, W, j, bytes);
+        uint32_t lo = 0, hi = 0;
+        if (ok) ok = enter_level(E.G, W, j, bytes, lo, hi);
         unsigned long long total = 0;
         unsigned long long wbase = WRITE ? E.off[r] - E.off[0] : 0;
         if (ok) {
-            const uint32_t lo = W.lo[j], hi = W.hi[j];
+            const uint4 C = W.C[j];
             for (uint32_t pos = lo; pos < hi; pos += 32) {
                 const uint32_t k = pos + lane;
                 int32_t c = -1;
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(ENUM_THREADS) k_extend(EnumPass E) {
                 uint32_t rej = 0;
                 if (k < hi) {
                     c = __ldg(E.G.adj + k);
-                    good = check_candidate(E.G, W, j, c, nullptr, probes, rej);
+                    good = check_candidate(E.G, W, C, j, c, nullptr, probes, rej);
                 }
                 const unsigned mask = __ballot_sync(FULLMASK, good);
                 scanned += min(32u, hi - pos);

@@ -11,6 +11,9 @@ struct DeviceGraph;  // resident CSR + label index + per-graph evaluation worksp
 struct EvalConfig {
     int32_t w_min = 32;         // speculation window per pattern (slots), lower bound
     int32_t w_max = 512;        // upper bound (hash table in shared memory sized for it)
+    bool streamed = false;      // the streaming greedy; no windows then
+    bool want_mni = true;       // some plan wants the MNI
+    bool cyclic = false;        // some pattern has a cycle (membership tests)
     int32_t search_blocks = 0;  // 0: SM count x resident blocks per SM
     int32_t record_selected = 0;
     int32_t rounds_per_sync = 4;
@@ -60,7 +63,7 @@ int dev_selected(DeviceGraph *g, int32_t i, int32_t *maps_out, int64_t cap, int6
 
 // Device bytes one pattern of a batch holds (used bitmap, two window buffers, items, state,
 // plan, result); and the device's free memory.
-int dev_pattern_bytes(const DeviceGraph *g, int32_t Wmax, int32_t sel, int64_t *bytes);
+int dev_pattern_bytes(const DeviceGraph *g, int32_t Wmax, int32_t sel, bool streamed, int64_t *bytes);
 
 // One pattern evaluated with device scratch taken from a static device array (no allocation).
 int dev_support_noalloc(DeviceGraph *g, const Plan *h_plan, flexis_support_result *h_out,

@@ -224,6 +224,136 @@ __global__ void k_gb_low(const unsigned long long *a, long long n, int32_t *out)
         out[i] = (int32_t)(uint32_t)a[i];
 }
 
+// Slice table: off[row * (nl + 1) + l] = adjacency position of the row's first neighbour with rank
+// label >= l, entry nl the row's end.  One warp per row: the labels present form a bit set, the
+// number of them below l is the run that entry l points at, and a row's entries are written
+// coalesced.  Bound by the writes (4 (nl + 1) bytes a row).
+__global__ void __launch_bounds__(GB_THREADS) k_slice_table(const VRec *vrec, const uint32_t *runs, long long rows,
+                                                            int nl, uint32_t *off) {
+    __shared__ uint32_t present[GB_THREADS / 32][8];
+    const int lane = threadIdx.x & 31;
+    uint32_t *pw = present[threadIdx.x >> 5];
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(vrec + r));
+        const uint32_t *ru = runs + v.y;
+        const uint32_t nrun = v.w >> 8;
+        if (lane < 8) pw[lane] = 0u;
+        __syncwarp();
+        for (uint32_t j = lane; j < nrun; j += 32) {
+            const uint32_t l = __ldg(ru + j) >> 24;
+            atomicOr(&pw[l >> 5], 1u << (l & 31));
+        }
+        __syncwarp();
+        uint32_t *o = off + r * (nl + 1);
+        uint32_t before = 0;  // labels present below this word's
+        for (int b = 0; b <= nl; b += 32) {
+            const uint32_t w = pw[b >> 5];
+            const int l = b + lane;
+            if (l <= nl) o[l] = v.x + (__ldg(ru + before + __popc(w & ((1u << lane) - 1u))) & 0xFFFFFFu);
+            before += __popc(w);
+        }
+        __syncwarp();
+    }
+}
+
+int dev_slice_table(DeviceGraph *g, int nl) {
+    const long long rows = g->vrec_count;
+    const int64_t bytes = 4ll * rows * (nl + 1);
+    size_t fr = 0, tot = 0;
+    CK(cudaMemGetInfo(&fr, &tot));
+    g->view.off = nullptr;
+    g->view.nl1 = nl + 1;
+    if (nl < 1 || g->view.nv < 1 || bytes > SLICE_TABLE_BYTES || bytes > (int64_t)(fr / 8)) return FLEXIS_OK;
+    CK(cudaMalloc(&g->d_off, (size_t)bytes));
+    g->bytes += bytes;
+    const long long want = (rows * 32 + GB_THREADS - 1) / GB_THREADS;
+    const int blocks = (int)std::min<long long>(want, (long long)std::max(1, g->sm_count) * 8);
+    k_slice_table<<<blocks, GB_THREADS, 0, g->stream>>>((const VRec *)g->d_vrec, (const uint32_t *)g->d_runs, rows, nl,
+                                                        (uint32_t *)g->d_off);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(g->stream));
+    g->view.off = (const uint32_t *)g->d_off;
+    return FLEXIS_OK;
+}
+
+static int bit_width(unsigned long long x) {
+    int b = 0;
+    while (x) {
+        b++;
+        x >>= 1;
+    }
+    return b;
+}
+
+// Edge set: a warp per row inserts the row's neighbours with a larger id.
+__global__ void __launch_bounds__(GB_THREADS) k_edge_set(DevGraphView G, uint32_t *table, unsigned int *failed) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < G.nv; v += nw) {
+        const uint4 r = __ldg(reinterpret_cast<const uint4 *>(G.vrec + v));
+        for (uint32_t k = lane; k < r.z; k += 32) {
+            const int32_t w = __ldg(G.adj + r.x + k);
+            if ((long long)w <= v) continue;
+            uint32_t bucket, entry;
+            edge_key(G, (uint32_t)v, (uint32_t)w, bucket, entry);
+            bool placed = false;
+            for (uint32_t d = 0; d < EDGE_DIST && !placed; d++) {
+                uint32_t *b = table + (size_t)((bucket + d) & G.eb_mask) * EDGE_WAYS;
+                for (int j = 0; j < EDGE_WAYS && !placed; j++)
+                    placed = __ldcg(b + j) == 0u && atomicCAS(b + j, 0u, entry | d << EDGE_DIST_SHIFT) == 0u;
+            }
+            if (!placed) atomicAdd(failed, 1u);
+        }
+    }
+}
+
+int dev_edge_set(DeviceGraph *g) {
+    if (g->edges_tried || g->view.dstride != 0 || g->view.nv < 2) return FLEXIS_OK;
+    g->edges_tried = true;
+    DevGraphView V = g->view;
+    V.eb_bits = bit_width((unsigned long long)V.nv - 1);
+    V.eb_log = std::max(5, 2 * V.eb_bits - (int)(EDGE_DIST_SHIFT - 1));
+    // three edges a bucket on average: one in 80 buckets is full
+    while ((3ll << V.eb_log) < g->n_arcs / 2) V.eb_log++;
+    const int64_t bytes = 4ll * EDGE_WAYS << V.eb_log;
+    size_t fr = 0, tot = 0;
+    CK(cudaMemGetInfo(&fr, &tot));
+    if (bytes > EDGE_SET_BYTES || bytes > (int64_t)(fr / 8) || V.eb_log >= 32) return FLEXIS_OK;
+    V.eb_mask = (uint32_t)((1ull << V.eb_log) - 1);
+    unsigned int *failed = nullptr, h = 0;
+    CK(cudaMalloc((void **)&failed, sizeof *failed));
+    auto done = [&](int rc) {
+        cudaFree(failed);
+        if (rc || h) {
+            cudaFree(g->d_edges);
+            g->d_edges = nullptr;
+        }
+        return rc;
+    };
+    if (cudaMalloc(&g->d_edges, (size_t)bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        g->d_edges = nullptr;
+        return done(FLEXIS_OK);
+    }
+    const int blocks = (int)std::min<long long>((V.nv * 32 + GB_THREADS - 1) / GB_THREADS,
+                                                (long long)std::max(1, g->sm_count) * 8);
+    if (cudaMemsetAsync(g->d_edges, 0, (size_t)bytes, g->stream) != cudaSuccess ||
+        cudaMemsetAsync(failed, 0, sizeof *failed, g->stream) != cudaSuccess)
+        return done(FLEXIS_E_CUDA);
+    k_edge_set<<<blocks, GB_THREADS, 0, g->stream>>>(V, (uint32_t *)g->d_edges, failed);
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemcpyAsync(&h, failed, sizeof h, cudaMemcpyDeviceToHost, g->stream) != cudaSuccess ||
+        cudaStreamSynchronize(g->stream) != cudaSuccess)
+        return done(FLEXIS_E_CUDA);
+    if (!h) {
+        V.edges = (const uint4 *)g->d_edges;
+        g->view = V;
+        g->bytes += bytes;
+    }
+    return done(FLEXIS_OK);
+}
+
 namespace {
 
 // Device temporaries of one build, freed on every exit.
@@ -239,15 +369,6 @@ struct Temps {
         for (void *q : p) cudaFree(q);
     }
 };
-
-int bit_width(unsigned long long x) {
-    int b = 0;
-    while (x) {
-        b++;
-        x >>= 1;
-    }
-    return b;
-}
 
 struct Sorter {
     cudaStream_t s;
@@ -440,6 +561,8 @@ int dev_graph_build(int64_t nv, const int32_t *labels, int64_t ne, const int32_t
     g->view.words = (int32_t)std::max<int64_t>(1, (nv + 31) / 32);
     g->view.dstride = 0;
     g->max_degree = hg.max_degree;
+    g->n_arcs = hg.n_arcs;
+    if ((rc = dev_slice_table(g, hg.nl))) return fail(rc);
     *out = g;
     return FLEXIS_OK;
 }

@@ -37,112 +37,12 @@
 #include <mutex>
 #include <vector>
 
-#include "fx_kern.cuh"
+#include "fx_stream.h"
 
 namespace fx {
 
-// window slot states.  A SEQ slot's root search ran out of its per-round budget: its remaining
-// search space is an ordered list of saved sub-searches (the first one's index in the slot's
-// map entry 0, each saved state holding the index of the next); the slot's map is the map of
-// the first sub-search in that order that finds one, once every earlier one has found none.
-enum : int32_t { SLOT_NEEDS = 0, SLOT_MAP = 1, SLOT_NONE = 2, SLOT_SEQ = 3 };
-// saved sub-search status (word SUSP_STATUS of its saved state); its map in SUSP_MAP..+7
-enum : int32_t { SS_PENDING = 0, SS_NONE = 1, SS_FOUND = 2 };
-constexpr int SPLIT_MAX = 15;  // pieces one split may create
-
-
-// slot phases: free, greedy rounds, MNI pending, result ready
-enum : int32_t { PH_FREE = 0, PH_GREEDY = 1, PH_MNI = 2, PH_READY = 3 };
-
-struct PatState {
-    int64_t count;     // maps selected so far
-    int64_t searched;  // root searches run
-    int32_t cursor;    // next root (index into lab_vtx)
-    int32_t nwin;      // slots in the window
-    int32_t W;         // target window size
-    int32_t done;
-    int32_t exhausted; // every root processed
-    int32_t rounds;
-    int32_t phase;
-    int32_t logged;    // selected maps written to the selection log
-    unsigned long long mni_cnt[MAXN];
-    unsigned long long steps;  // candidate chunks scanned by the greedy searches
-    uint32_t max_steps;        // largest chunk count of one greedy search
-    int32_t buf;               // current window buffer (0 or 1)
-    uint32_t susp_mask;        // saved-search slots in use (KSUSP bits)
-    uint32_t cancelled;        // stopped at a deadline before its decision
-    uint32_t mni_cut;          // the MNI pass passed the deadline before this pattern's count
-    int32_t ndirty;            // used-bitmap words this pattern made non-zero (listed up to DIRTY_CAP)
-};
-
-struct Ctl {
-    int32_t n_items[2];
-    int32_t next_item[2];
-    int32_t active[2];
-    int32_t acount[2];    // lengths of the two active-pattern lists
-    int32_t idle[2];      // warps of the search launch that found no work item left
-    int32_t drain[2];     // set once idle reaches the launch's drain threshold
-    int32_t err;
-    int32_t pad;
-    unsigned long long bytes_greedy;
-    unsigned long long bytes_mni;
-    unsigned long long alg_scanned;   // greedy search: driver-slice entries scanned (A)
-    unsigned long long alg_bound;     // greedy search: sum over bound partial maps of their length
-    unsigned long long alg_map_words; // greedy search: words of the maps it wrote (n per map found)
-    unsigned long long search_items;
-    unsigned long long mni_items;
-    unsigned long long mni_total;
-    unsigned long long mni_next;
-    unsigned long long t0_ns;     // device clock at the start of the evaluation (k_init)
-};
-
-struct Batch {
-    DevGraphView G;
-    const Plan *plans;
-    int32_t P;
-    int32_t Wmax;
-    int32_t Wmin;
-    int32_t sel_cap;
-    uint32_t budget;      // per-round candidate chunks of one root search (0: unlimited)
-    int32_t split_max;    // pieces per split (0: no split)
-    uint32_t sid_all;     // saved sub-search indices a pattern may use (bit set)
-    PatState *st;
-    uint32_t *used;       // [P][words]
-    int32_t *dirty;       // [P][DIRTY_CAP] words of `used` made non-zero (nullable: not tracked)
-    int32_t *win_root;    // [P][2][Wmax]  two window buffers per pattern
-    int32_t *win_state;   // [P][2][Wmax]
-    int32_t *win_map;     // [P][2][Wmax][8] (by level)
-    int2 *items;          // [P*Wmax] (pattern, buffer * Wmax + slot)
-    Ctl *ctl;
-    int32_t *sel;         // [P][sel_cap][8] selected maps, canonical vertex order
-    unsigned long long *mni_seg;  // [P*8+1] prefix sums of MNI candidate segments
-    int32_t *alist;               // [2][P] patterns still in their greedy phase (nullable: all)
-    uint32_t *susp;               // [P][KSUSP][DFS_SAVE_STRIDE] saved search states
-    flexis_support_result *results;
-    unsigned long long deadline_ns;  // > 0: the MNI pass stops this long after ctl->t0_ns
-};
-
-// The device's global nanosecond clock (PTX special register %globaltimer).
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-constexpr int DFS_SAVE_WORDS = (int)(offsetof(WarpState, need) / 4);
-constexpr int DFS_SAVE_STRIDE = 192;  // words per saved sub-search
-constexpr int SUSP_STATUS = DFS_SAVE_WORDS;      // SS_* of the saved sub-search
-constexpr int SUSP_NEXT = DFS_SAVE_WORDS + 1;    // next sub-search of the same slot, or -1
-constexpr int SUSP_MAP = DFS_SAVE_WORDS + 2;     // its map (by level) when SS_FOUND
-static_assert(SUSP_MAP + MAXN <= DFS_SAVE_STRIDE, "saved search state too large");
-constexpr int KSUSP = 32;             // saved sub-searches a pattern may hold at once
-constexpr uint32_t SEARCH_BUDGET = 4096;  // candidate chunks a root search runs per round
-
-
 // ------------------------------------------------------------------ kernels
-constexpr int SEARCH_THREADS = 256;
 constexpr int DRAIN_DIV = 8;  // the searches drain once all but 1/DRAIN_DIV of the launch's warps are idle
-constexpr int DIRTY_CAP = 1024;  // listed used-bitmap words per pattern (4 KB)
 constexpr int COMMIT_THREADS = 256;
 
 __device__ void reset_ctl(Ctl *c) {
@@ -227,7 +127,7 @@ __device__ __forceinline__ void save_state(uint32_t *dst, const WarpState &W, in
 // eighth of the launch's warps have found the item list empty, the searches still running are
 // saved (and split) the same way at their next drain check instead of running to the budget,
 // so a launch is not held open by a few long searches while most of the GPU idles.
-__global__ void __launch_bounds__(SEARCH_THREADS, 6) k_search(Batch B, int q) {
+__global__ void __launch_bounds__(SEARCH_THREADS, 4) k_search(Batch B, int q) {
     __shared__ WarpState ws[SEARCH_THREADS / 32];
     const int lane = threadIdx.x & 31;
     WarpState &W = ws[threadIdx.x >> 5];
@@ -256,11 +156,12 @@ __global__ void __launch_bounds__(SEARCH_THREADS, 6) k_search(Batch B, int q) {
         const int off = item.y & 0xFFFFFF;
         const int sid_in = (item.y >> 24) - 1;
         const Plan &P = B.plans[p];
-        const size_t slot = (size_t)p * 2 * B.Wmax + off;
+        const size_t h = (size_t)p;
+        const size_t slot = h * 2 * B.Wmax + off;
         int32_t *seq = B.win_map + slot * MAXN;
         const int32_t root = B.win_root[slot];
-        const uint32_t *used = B.used + (size_t)p * B.G.words;
-        uint32_t *sbase = B.susp + (size_t)p * KSUSP * DFS_SAVE_STRIDE;
+        const uint32_t *used = B.used + h * B.G.words;
+        uint32_t *sbase = B.susp + h * KSUSP * DFS_SAVE_STRIDE;
         const bool resume = sid_in >= 0;
         load_level_plan(W, P.greedy, P);
         if (resume) {
@@ -269,7 +170,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, 6) k_search(Batch B, int q) {
             __syncwarp();
         }
         uint32_t steps = 0;
-        int r = dfs_run(B.G, W, used, root, bytes, probes, steps, B.budget, resume, work, &B.ctl->drain[q]);
+        int r = dfs_run(B.G, W, used, root, bytes, probes, steps, resume, work, BudgetStop{B.budget, &B.ctl->drain[q]});
         if (lane == 0) {
             W.acc_scanned += work.scanned;
             W.acc_bound += work.bound;
@@ -421,12 +322,13 @@ __device__ __forceinline__ void commit_one(const Batch &B, int q, int p, int32_t
     const int nwin = S->nwin;
     const int Wmax = B.Wmax;
     const int cur = S->buf, nxt = cur ^ 1;
-    const size_t pb = (size_t)p * 2 * Wmax;
+    const size_t h = (size_t)p;
+    const size_t pb = h * 2 * Wmax;
     const size_t cb = pb + (size_t)cur * Wmax, nb = pb + (size_t)nxt * Wmax;
     const int32_t *st_cur = B.win_state + cb, *rt_cur = B.win_root + cb, *mp_cur = B.win_map + cb * MAXN;
     int32_t *st_nxt = B.win_state + nb, *rt_nxt = B.win_root + nb, *mp_nxt = B.win_map + nb * MAXN;
-    uint32_t *used = B.used + (size_t)p * B.G.words;
-    uint32_t *sbase = B.susp + (size_t)p * KSUSP * DFS_SAVE_STRIDE;
+    uint32_t *used = B.used + h * B.G.words;
+    uint32_t *sbase = B.susp + h * KSUSP * DFS_SAVE_STRIDE;
 
     // 0. sub-search sequences: drop sub-searches that found nothing; a slot whose first
     //    remaining sub-search found a map takes that map (if a vertex of it has been used since,
@@ -551,7 +453,7 @@ __device__ __forceinline__ void commit_one(const Batch &B, int q, int p, int32_t
                 const uint32_t old = atomicOr(used + wi, 1u << (m[l] & 31));
                 if (old == 0 && B.dirty) {  // first bit of this word: list it for the clean-up
                     const int k = atomicAdd(&S->ndirty, 1);
-                    if (k < DIRTY_CAP) B.dirty[(size_t)p * DIRTY_CAP + k] = (int32_t)wi;
+                    if (k < DIRTY_CAP) B.dirty[h * DIRTY_CAP + k] = (int32_t)wi;
                 }
             }
             const int64_t at = count0 + ncommit + excl;
@@ -757,7 +659,7 @@ constexpr int MNI_CHUNK = 8;
 constexpr uint32_t MNI_BUDGET = 4096;  // candidate chunks of an MNI search between deadline checks
 
 // One warp per candidate vertex d of an orbit: does some map send the orbit representative to d?
-__global__ void __launch_bounds__(SEARCH_THREADS) k_mni(Batch B) {
+__global__ void __launch_bounds__(SEARCH_THREADS, 4) k_mni(Batch B) {
     __shared__ WarpState ws[SEARCH_THREADS / 32];
     const int lane = threadIdx.x & 31;
     WarpState &W = ws[threadIdx.x >> 5];
@@ -795,14 +697,15 @@ __global__ void __launch_bounds__(SEARCH_THREADS) k_mni(Batch B) {
             // existence search in slices of MNI_BUDGET candidate chunks; between slices the
             // deadline is checked and the search resumes where it stopped
             SearchWork work;
-            int r = dfs_run(B.G, W, nullptr, d, bytes, probes, steps, MNI_BUDGET, false, work);
-            while (r == DFS_SUSPENDED) {
+            int r;
+            for (bool again = false;; again = true) {
+                steps = 0;
+                r = dfs_run(B.G, W, nullptr, d, bytes, probes, steps, again, work, BudgetStop{MNI_BUDGET, nullptr});
+                if (r != DFS_SUSPENDED) break;
                 if (B.deadline_ns && global_ns() - B.ctl->t0_ns > B.deadline_ns) {
                     if (lane == 0) B.st[p].mni_cut = 1u;
                     break;
                 }
-                steps = 0;
-                r = dfs_run(B.G, W, nullptr, d, bytes, probes, steps, MNI_BUDGET, true, work);
             }
             scanned_all += work.scanned;
             if (r == DFS_FOUND && lane == 0) atomicAdd(cnt, 1ull);
@@ -840,7 +743,7 @@ __global__ void k_clear_used(Batch B) {
     const int nd = B.st[p].ndirty;
     if (nd <= DIRTY_CAP) {
         const int32_t *d = B.dirty + (size_t)p * DIRTY_CAP;
-        for (int i = lane; i < nd; i += 32) u[d[i]] = 0u;
+        for (int k = lane; k < nd; k += 32) u[d[k]] = 0u;
     } else {
         for (uint32_t w = lane; w < B.G.words; w += 32) u[w] = 0u;
     }
@@ -931,7 +834,12 @@ template <int KM>
 static size_t commit_smem_of() { return sizeof(int32_t) * 2 * commit_hash<KM>(); }
 static size_t commit_smem(int) { return commit_smem_of<KMAP>(); }
 
-int dev_pattern_bytes(const DeviceGraph *g, int32_t Wmax, int32_t sel, int64_t *bytes) {
+int dev_pattern_bytes(const DeviceGraph *g, int32_t Wmax, int32_t sel, bool streamed, int64_t *bytes) {
+    if (streamed) {  // bitmaps and windows are held per slot, not per pattern
+        *bytes = (int64_t)sizeof(PatState) + (int64_t)sizeof(Plan) + (int64_t)sizeof(flexis_support_result) +
+                 8 * MAXN + 12 + (int64_t)sel * 4 * MAXN;
+        return FLEXIS_OK;
+    }
     *bytes = (int64_t)g->view.words * 4 + 4ll * DIRTY_CAP + (int64_t)Wmax * (2 * (4 + 4 + 4 * MAXN) + 8) + 8 * KSUSP +
              (int64_t)sizeof(PatState) + (int64_t)sizeof(Plan) + (int64_t)sizeof(flexis_support_result) +
              8 * (MAXN + 1) + (int64_t)sel * 4 * MAXN + 4ll * KSUSP * DFS_SAVE_STRIDE;
@@ -942,7 +850,7 @@ int dev_free_bytes(const DeviceGraph *g, int64_t *bytes) {
     size_t fr = 0, tot = 0;
     CK(cudaSetDevice(g->device));
     CK(cudaMemGetInfo(&fr, &tot));
-    *bytes = (int64_t)std::min(fr + (size_t)g->ws.bytes, tot);  // free + what the workspace holds
+    *bytes = (int64_t)std::min(fr + (size_t)g->ws.bytes + (size_t)g->sws.bytes, tot);  // free + what the workspaces hold
     return FLEXIS_OK;
 }
 
@@ -969,6 +877,7 @@ int dev_graph_init(int device, DeviceGraph **out) {
                                                           commit_smem_of<KMAP_SMALL>()) != cudaSuccess)
             per_sm = 1;
         g->commit_small_blocks = g->sm_count * std::max(1, per_sm);
+        g->stream_per_sm = stream_blocks_per_sm();
     }
     *out = g;
     return FLEXIS_OK;
@@ -997,6 +906,8 @@ int dev_graph_create(const HostGraph &hg, int device, DeviceGraph **out) {
     g->view.words = (int32_t)std::max<int64_t>(1, (hg.nv + 31) / 32);
     g->view.dstride = hg.directed ? hg.nv : 0;
     g->max_degree = hg.max_degree;
+    g->n_arcs = hg.n_arcs;
+    if ((rc = dev_slice_table(g, hg.nl))) return fail(rc);
     *out = g;
     return FLEXIS_OK;
 }
@@ -1012,15 +923,16 @@ static void ws_free(Workspace &w) {
 // Capacity is kept in patterns and in window slots (patterns x Wmax) separately, so a large
 // batch with small windows followed by a small batch with large windows never allocates the
 // product of the two.
-static int ws_ensure(DeviceGraph *g, Workspace &w, int32_t P, int32_t Wmax, int32_t sel) {
-    const int64_t slots = (int64_t)P * Wmax;
-    if (P <= w.P && slots <= w.slots && (int64_t)P * sel <= w.sel_slots && w.h_ctl) return FLEXIS_OK;
+static int ws_ensure(DeviceGraph *g, Workspace &w, int32_t P, int32_t H, int32_t Wmax, int32_t sel) {
+    const int64_t slots = (int64_t)H * Wmax;
+    if (P <= w.P && H <= w.H && slots <= w.slots && (int64_t)P * sel <= w.sel_slots && w.h_ctl) return FLEXIS_OK;
     const int32_t nP = std::max(P, w.P);
+    const int32_t nH = std::max(H, w.H);
     const int64_t nSlots = std::max(slots, w.slots);
     const int64_t nSel = std::max((int64_t)P * sel, w.sel_slots);
-    // the captured round loop holds the old buffers' addresses: it goes with them
-    if (&w == &g->ws && g->round_exec) {
-        cudaGraphExecDestroy(g->round_exec);
+    // the captured launches hold the old buffers' addresses: they go with them
+    if (&w == &g->ws) {
+        if (g->round_exec) cudaGraphExecDestroy(g->round_exec);
         g->round_exec = nullptr;
     }
     ws_free(w);
@@ -1031,24 +943,62 @@ static int ws_ensure(DeviceGraph *g, Workspace &w, int32_t P, int32_t Wmax, int3
         return cudaMalloc(ptr, std::max<size_t>(bytes, 16));
     };
     CK(alloc((void **)&w.st, sizeof(PatState) * nP));
-    CK(alloc((void **)&w.used, sizeof(uint32_t) * words * nP));
-    CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nP));
+    CK(alloc((void **)&w.used, sizeof(uint32_t) * words * nH));
+    CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nH));
     w.clean = 0;
     CK(alloc((void **)&w.win_root, sizeof(int32_t) * (size_t)nSlots * 2));
     CK(alloc((void **)&w.win_state, sizeof(int32_t) * (size_t)nSlots * 2));
     CK(alloc((void **)&w.win_map, sizeof(int32_t) * (size_t)nSlots * 2 * MAXN));
-    CK(alloc((void **)&w.items, sizeof(int2) * ((size_t)nSlots + (size_t)nP * KSUSP)));
+    CK(alloc((void **)&w.items, sizeof(int2) * ((size_t)nSlots + (size_t)nH * KSUSP)));
     CK(alloc((void **)&w.ctl, sizeof(Ctl)));
     CK(alloc((void **)&w.mni_seg, sizeof(unsigned long long) * ((size_t)nP * MAXN + 1)));
-    CK(alloc((void **)&w.susp, sizeof(uint32_t) * (size_t)nP * KSUSP * DFS_SAVE_STRIDE));
+    CK(alloc((void **)&w.susp, sizeof(uint32_t) * (size_t)nH * KSUSP * DFS_SAVE_STRIDE));
     CK(alloc((void **)&w.alist, sizeof(int32_t) * (size_t)nP * 2));
     CK(alloc((void **)&w.plans, sizeof(Plan) * (size_t)nP));
     CK(alloc((void **)&w.results, sizeof(flexis_support_result) * (size_t)nP));
     if (nSel > 0) CK(alloc((void **)&w.sel_buf, sizeof(int32_t) * (size_t)nSel * MAXN));
     CK(cudaMallocHost((void **)&w.h_ctl, sizeof(Ctl)));
     w.P = nP;
+    w.H = nH;
     w.slots = nSlots;
     w.sel_slots = nSel;
+    w.bytes = b;
+    return FLEXIS_OK;
+}
+
+static void sws_free(StreamWS &w) {
+    cudaFree(w.words); cudaFree(w.slots); cudaFree(w.status); cudaFree(w.mask); cudaFree(w.used);
+    cudaFree(w.maps); cudaFree(w.dirty); cudaFree(w.dead);
+    cudaFree(w.tasks); cudaFree(w.task_links); cudaFree(w.teams);
+    w = StreamWS();
+}
+
+static int sws_ensure(DeviceGraph *g, int32_t S, int64_t ring) {
+    StreamWS &w = g->sws;
+    if (S <= w.S && ring <= w.ring) return FLEXIS_OK;
+    const int32_t nS = std::max(S, w.S);
+    const int64_t nR = std::max(ring, w.ring);
+    if (g->stream_exec) cudaGraphExecDestroy(g->stream_exec);
+    g->stream_exec = nullptr;
+    sws_free(w);
+    int64_t b = 0;
+    auto alloc = [&](void **ptr, size_t bytes) {
+        b += (int64_t)bytes;
+        return cudaMalloc(ptr, bytes);
+    };
+    CK(alloc((void **)&w.words, sizeof(unsigned long long) * (size_t)nS));
+    CK(alloc((void **)&w.slots, sizeof(StreamSlot) * (size_t)nS));
+    CK(alloc((void **)&w.status, sizeof(uint32_t) * (size_t)(nR / STREAM_GS_MIN)));
+    CK(alloc((void **)&w.mask, sizeof(uint32_t) * (size_t)(nR / STREAM_GS_MIN) * 2));
+    CK(alloc((void **)&w.maps, sizeof(int32_t) * (size_t)nR * MAXN));
+    CK(alloc((void **)&w.used, sizeof(uint32_t) * (size_t)g->view.words * nS));
+    CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nS));
+    CK(alloc((void **)&w.tasks, sizeof(uint32_t) * (size_t)STREAM_TASKS * STREAM_TASK_WORDS));
+    CK(alloc((void **)&w.task_links, sizeof(int32_t) * (size_t)(3 * STREAM_TASKS + STREAM_TEAMS)));
+    CK(alloc((void **)&w.teams, (size_t)STREAM_TEAMS * STREAM_TEAM_BYTES));
+    CK(alloc((void **)&w.dead, sizeof(uint32_t) * ((size_t)nS << DEAD_LOG)));
+    w.S = nS;
+    w.ring = nR;
     w.bytes = b;
     return FLEXIS_OK;
 }
@@ -1058,12 +1008,14 @@ void dev_graph_destroy(DeviceGraph *g) {
     cudaSetDevice(g->device);
     if (g->stream) cudaStreamSynchronize(g->stream);
     ws_free(g->ws);
+    sws_free(g->sws);
     enum_ws_destroy(g);
-    cudaFree(g->d_vrec); cudaFree(g->d_runs); cudaFree(g->d_adj); cudaFree(g->d_labvtx);
+    cudaFree(g->d_vrec); cudaFree(g->d_runs); cudaFree(g->d_adj); cudaFree(g->d_labvtx); cudaFree(g->d_off); cudaFree(g->d_edges);
     if (g->ev[0]) cudaEventDestroy(g->ev[0]);
     if (g->ev[1]) cudaEventDestroy(g->ev[1]);
     for (auto e : g->sev) cudaEventDestroy(e);
     if (g->round_exec) cudaGraphExecDestroy(g->round_exec);
+    if (g->stream_exec) cudaGraphExecDestroy(g->stream_exec);
     for (auto e : g->gev) cudaEventDestroy(e);
     if (g->stream) cudaStreamDestroy(g->stream);
     delete g;
@@ -1137,10 +1089,6 @@ static int search_grid(const DeviceGraph *g, const EvalConfig &cfg) {
     return cfg.search_blocks > 0 ? cfg.search_blocks : g->sm_count * std::max(1, per_sm);
 }
 
-// Capture R rounds (commit + search, alternating window buffers from 0) and the control-word
-// read into g->round_exec, updating the executable graph in place when only the kernel
-// parameters changed.  Returns 0 on success; on any failure the stream is left out of capture,
-// the error is cleared, and the caller launches the kernels one by one.
 static void launch_commit(const Batch &B, int q, bool small, int commit_blocks, size_t smem, cudaStream_t stream) {
     if (small)
         k_commit<KMAP_SMALL><<<commit_blocks, COMMIT_THREADS_SMALL, smem, stream>>>(B, q);
@@ -1152,23 +1100,17 @@ static void launch_search(const Batch &B, int q, int sblocks, cudaStream_t strea
     k_search<<<sblocks, SEARCH_THREADS, 0, stream>>>(B, q);
 }
 
-static int capture_rounds(DeviceGraph *g, const Batch &B, int R, bool small, int commit_blocks, size_t smem,
-                          int sblocks, cudaStream_t stream, Ctl *h_ctl, Ctl *d_ctl,
-                          const cudaEvent_t *tev) {
+// Capture what `body` launches on `stream` into *exec, updating the executable graph in place when
+// only parameters changed.  Returns 0 on success; on any failure the stream is left out of
+// capture, the error is cleared, and the caller launches directly.
+template <class F>
+static int capture_graph(DeviceGraph *g, cudaGraphExec_t *exec, cudaStream_t stream, F body) {
     cudaGraph_t gr = nullptr;
     if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         (void)cudaGetLastError();
         return 1;
     }
-    for (int r = 0; r < R; r++) {
-        launch_commit(B, r & 1, small, commit_blocks, smem, stream);
-        // an event record node needs the external flag (a plain record inside a capture only
-        // orders streams)
-        if (tev) cudaEventRecordWithFlags(tev[2 * r], stream, cudaEventRecordExternal);
-        launch_search(B, r & 1, sblocks, stream);
-        if (tev) cudaEventRecordWithFlags(tev[2 * r + 1], stream, cudaEventRecordExternal);
-    }
-    cudaMemcpyAsync(h_ctl, d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+    body();
     const cudaError_t ce = cudaStreamEndCapture(stream, &gr);
     if (ce != cudaSuccess || gr == nullptr) {
         if (gr) cudaGraphDestroy(gr);
@@ -1176,25 +1118,143 @@ static int capture_rounds(DeviceGraph *g, const Batch &B, int R, bool small, int
         return 1;
     }
     bool ok = false;
-    if (g->round_exec) {
+    if (*exec) {
         cudaGraphExecUpdateResultInfo info;
-        ok = cudaGraphExecUpdate(g->round_exec, gr, &info) == cudaSuccess;
+        ok = cudaGraphExecUpdate(*exec, gr, &info) == cudaSuccess;
         if (!ok) {
             (void)cudaGetLastError();
-            cudaGraphExecDestroy(g->round_exec);
-            g->round_exec = nullptr;
+            cudaGraphExecDestroy(*exec);
+            *exec = nullptr;
         }
     }
     if (!ok) {
-        ok = cudaGraphInstantiate(&g->round_exec, gr, 0) == cudaSuccess;
+        ok = cudaGraphInstantiate(exec, gr, 0) == cudaSuccess;
         if (!ok) {
             (void)cudaGetLastError();
-            g->round_exec = nullptr;
+            *exec = nullptr;
         }
         g->graph_instantiations += ok;
     }
     cudaGraphDestroy(gr);
     return ok ? 0 : 1;
+}
+
+// What an evaluation did, for the stats.
+struct EvalCounts {
+    int64_t launches = 0, rounds = 0, graph_launches = 0;
+    int search_launches = 0, reads = 0;
+    float search_ms = 0.f;
+    bool timed_out = false;
+};
+
+static int timing_events(std::vector<cudaEvent_t> &v, size_t n) {
+    while (v.size() < n) {
+        cudaEvent_t e;
+        CK(cudaEventCreate(&e));
+        v.push_back(e);
+    }
+    return FLEXIS_OK;
+}
+
+// The windowed rounds: commit and search kernels until no pattern of the batch is active (or the
+// deadline passes: the undecided patterns are then stopped).
+static int run_rounds(DeviceGraph *g, Workspace &w, const Batch &B, const EvalConfig &cfg, bool small_commit,
+                      int commit_blocks, cudaStream_t stream, bool use_graph,
+                      std::chrono::steady_clock::time_point t_start, EvalCounts &c) {
+    const size_t smem = small_commit ? commit_smem_of<KMAP_SMALL>() : commit_smem(B.Wmax);
+    const int sblocks = search_grid(g, cfg);
+    int R = std::max(1, cfg.rounds_per_sync);
+    if (use_graph) R += R & 1;
+    int64_t rounds = 0;
+    // the deadline is checked where the host waits anyway (between groups of rounds)
+    auto past_deadline = [&]() {
+        if (cfg.deadline_ms <= 0) return false;
+        const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
+        c.timed_out = ms > cfg.deadline_ms;
+        return c.timed_out;
+    };
+    if (cfg.timing)
+        if (int rc = timing_events(g->gev, (size_t)(2 * R))) return rc;
+    // With timing, an event pair brackets every search launch; the pairs are read after every group
+    // of rounds.  An event record node needs the external flag (a plain record inside a capture
+    // only orders streams).
+    auto launch_rounds = [&](bool captured) {
+        for (int r = 0; r < R; r++) {
+            const int q = (int)((rounds + r) & 1);
+            launch_commit(B, q, small_commit, commit_blocks, smem, stream);
+            if (cfg.timing) cudaEventRecordWithFlags(g->gev[2 * r], stream, captured ? cudaEventRecordExternal : cudaEventRecordDefault);
+            launch_search(B, q, sblocks, stream);
+            if (cfg.timing) cudaEventRecordWithFlags(g->gev[2 * r + 1], stream, captured ? cudaEventRecordExternal : cudaEventRecordDefault);
+        }
+        cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+    };
+    // The R rounds between two host checks (and the control-word read) are captured once into a
+    // CUDA graph and replayed.  R is even then, so that the window buffer parity of a replay matches
+    // the rounds it stands for.
+    const bool captured = use_graph && !capture_graph(g, &g->round_exec, stream, [&] { launch_rounds(true); });
+    if (use_graph && !captured) g->graph_fallbacks++;
+    for (;;) {
+        if (captured) {
+            CK(cudaGraphLaunch(g->round_exec, stream));
+            c.graph_launches++;
+        } else {
+            launch_rounds(false);
+            CK(cudaGetLastError());
+        }
+        c.launches += 2 * R;
+        c.search_launches += R;
+        c.reads++;
+        rounds += R;
+        CK(cudaStreamSynchronize(stream));
+        if (cfg.timing)
+            for (int r = 0; r < R; r++) {
+                float x = 0.f;
+                CK(cudaEventElapsedTime(&x, g->gev[2 * r], g->gev[2 * r + 1]));
+                c.search_ms += x;
+            }
+        if (w.h_ctl->active[(rounds - 1) & 1] == 0) break;
+        if (past_deadline()) break;
+    }
+    c.rounds += rounds;
+    if (c.timed_out) {
+        k_cancel<<<(B.P + 255) / 256, 256, 0, stream>>>(B, nullptr, B.P);
+        c.launches += 1;
+    }
+    return FLEXIS_OK;
+}
+
+static void launch_mni_finalize(const Batch &B, const EvalConfig &cfg, int sblocks, cudaStream_t stream,
+                                const cudaEvent_t *ev, unsigned flags, int64_t &launches) {
+    if (cfg.want_mni) {
+        k_mni_setup<<<1, 1024, 0, stream>>>(B);
+        if (ev) cudaEventRecordWithFlags(ev[0], stream, flags);
+        k_mni<<<sblocks, SEARCH_THREADS, 0, stream>>>(B);
+        if (ev) cudaEventRecordWithFlags(ev[1], stream, flags);
+        launches += 2;
+    }
+    k_finalize<<<(B.P + 255) / 256, 256, 0, stream>>>(B);
+    launches += 1;
+}
+
+// Slots, ring and group sizes of the streaming greedy for P patterns.
+static void stream_shape(const DeviceGraph *g, const EvalConfig &cfg, int32_t P, StreamArgs &A, int &blocks) {
+    constexpr int warps_per_block = SEARCH_THREADS / 32;
+    const int64_t bitmap = 4ll * g->view.words;
+    const int full = cfg.search_blocks > 0 ? cfg.search_blocks : g->sm_count * g->stream_per_sm;
+    // slots: one a warp when patterns are many (no map is ever stale then), never more than the warps
+    int64_t S = std::min<int64_t>({(int64_t)P, (int64_t)full * warps_per_block,
+                                   std::max<int64_t>(64, STREAM_BITMAP_BYTES / std::max<int64_t>(bitmap, 1))});
+    S = std::max<int64_t>(1, S);
+    A.S = (int32_t)S;
+    // groups: a lane a root when a warp has a pattern to itself; smaller ones the more warps share one
+    const int64_t wps = (int64_t)full * warps_per_block / S;
+    A.GS = wps <= 2 ? 32 : wps <= 8 ? 16 : 8;
+    int64_t rw = STREAM_RING_SLOT_MIN;
+    while (rw * 2 <= STREAM_RING_SLOT_MAX && rw * 2 * S <= STREAM_RING_ROOTS) rw *= 2;  // (a power of two)
+    A.RG = (int32_t)(rw / A.GS);
+    // at most STREAM_SLOT_WARPS warps a slot: more only get in each other's way
+    blocks = (int)std::min<int64_t>(full, std::max<int64_t>(1, S * STREAM_SLOT_WARPS / warps_per_block));
+    A.window0 = std::max(2, (S >= 128 ? 64 : 128) / A.GS);
 }
 
 int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_result *d_results,
@@ -1204,140 +1264,133 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
     CK(cudaSetDevice(g->device));
     const int Wmax = std::max(32, std::min(cfg.w_max, 16384));
     const int Wmin = std::max(1, std::min(cfg.w_min, Wmax));
-    int rc = ws_ensure(g, g->ws, P, Wmax, cfg.record_selected);
+    if (cfg.cyclic)
+        if (int rc = dev_edge_set(g)) return rc;
+    const bool streamed = cfg.streamed;
+    const int32_t H = streamed ? 0 : P;  // the streaming greedy has bitmaps of its own and no windows
+    int rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected);
     if (rc) return rc;
     Workspace &w = g->ws;
+    StreamArgs A{};
+    int stream_blocks = 0;
+    if (streamed) {
+        stream_shape(g, cfg, P, A, stream_blocks);
+        if ((rc = sws_ensure(g, A.S, (int64_t)A.S * A.RG * A.GS))) return rc;
+    }
+    StreamWS &sw = g->sws;
     g->last_P = P;
     g->last_sel = cfg.record_selected;
     Batch B = make_batch(g, w, d_plans, P, Wmin, Wmax, cfg.record_selected, d_results);
-    // large batches walk a list of the patterns still active; small ones launch a block per slot
-    const int list_threshold = 4 * g->sm_count;
-    if (P > list_threshold) B.alist = w.alist;
-    // large batches with windows of <= 1024 slots: the small-horizon commit, one full wave
-    const bool small_commit = P > list_threshold && Wmax <= SMALL_COMMIT_WMAX;
-    const int commit_blocks = small_commit ? g->commit_small_blocks : P > list_threshold ? list_threshold : P;
     if (cfg.search_budget != 0) B.budget = cfg.search_budget < 0 ? 0u : (uint32_t)cfg.search_budget;
     if (cfg.split_pieces != 0) B.split_max = cfg.split_pieces < 0 ? 0 : std::min(cfg.split_pieces, SPLIT_MAX);
     if (cfg.sub_searches > 0) {
         const int k = std::min(cfg.sub_searches, KSUSP);
         B.sid_all = k >= 32 ? 0xFFFFFFFFu : ((1u << k) - 1u);
     }
-    const size_t smem = small_commit ? commit_smem_of<KMAP_SMALL>() : commit_smem(Wmax);
     const int sblocks = search_grid(g, cfg);
     B.deadline_ns = cfg.deadline_ms > 0 ? (unsigned long long)cfg.deadline_ms * 1000000ull : 0ull;
+    const bool use_graph = cfg.graphs && stream != nullptr && stream != cudaStreamLegacy &&
+                           stream != cudaStreamPerThread;
+    const int list_threshold = 4 * g->sm_count;
+    EvalCounts c;
+    cudaEvent_t *mev = nullptr, *tev = nullptr;  // with timing: around the MNI and the stream kernel
+    if (cfg.timing) {
+        if ((rc = timing_events(g->sev, 4))) return rc;
+        mev = g->sev.data();
+        tev = g->sev.data() + 2;
+    }
+    float mni_ms = 0.f;
+    auto add_mni = [&]() {
+        float y = 0.f;
+        if (mev && cfg.want_mni && cudaEventElapsedTime(&y, mev[0], mev[1]) == cudaSuccess) mni_ms += y;
+    };
 
-    int64_t launches = 0;
     CK(cudaEventRecord(g->ev[0], stream));
     // used bitmaps: only those not known to be zero are cleared here (the previous evaluation
     // cleaned up after itself); until this one cleans up, none is known to be zero
     const int32_t clean0 = w.clean;
     w.clean = 0;
-    if (clean0 < P)
+    if (clean0 < H)
         CK(cudaMemsetAsync(w.used + (size_t)g->view.words * clean0, 0,
-                           sizeof(uint32_t) * (size_t)g->view.words * (P - clean0), stream));
-    CK(cudaMemsetAsync(w.ctl, 0, sizeof(Ctl), stream));
-    k_init<<<(P + 255) / 256, 256, 0, stream>>>(B);
-    launches += 1;
-    int64_t rounds = 0;
-    int search_launches = 0;
-    int R = std::max(1, cfg.rounds_per_sync);
-    size_t evi = 0;
-    // The R rounds between two host checks (commit + search each, then the control-word read)
-    // are captured once per level into a CUDA graph and replayed: the round loop's launches
-    // cost one graph launch per R rounds.  R is even so that the window buffer parity of a
-    // replay matches the rounds it stands for.
-    // With timing, the graph also records an event pair around each search launch; the pairs
-    // are read after every replay.
-    const bool use_graph = cfg.graphs && stream != nullptr && stream != cudaStreamLegacy &&
-                           stream != cudaStreamPerThread;
-    bool graph_done = false;
-    int64_t graph_launches = 0;
-    float graph_search_ms = 0.f;
-    // the deadline is checked where the host waits anyway (between groups of rounds)
-    bool timed_out = false;
-    auto past_deadline = [&]() {
-        if (cfg.deadline_ms <= 0) return false;
-        const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
-        timed_out = ms > cfg.deadline_ms;
-        return timed_out;
-    };
-    if (use_graph) {
-        R += R & 1;
-        while (cfg.timing && g->gev.size() < (size_t)(2 * R)) {
-            cudaEvent_t e;
-            CK(cudaEventCreate(&e));
-            g->gev.push_back(e);
+                           sizeof(uint32_t) * (size_t)g->view.words * (H - clean0), stream));
+    if (streamed) {
+        if (!sw.clean) {
+            CK(cudaMemsetAsync(sw.words, 0, sizeof(unsigned long long) * (size_t)sw.S, stream));
+            CK(cudaMemsetAsync(sw.status, 0, sizeof(uint32_t) * (size_t)(sw.ring / STREAM_GS_MIN), stream));
+            CK(cudaMemsetAsync(sw.used, 0, sizeof(uint32_t) * (size_t)g->view.words * sw.S, stream));
+            CK(cudaMemsetAsync(sw.dead, 0, sizeof(uint32_t) * ((size_t)sw.S << DEAD_LOG), stream));
         }
-        if (!capture_rounds(g, B, R, small_commit, commit_blocks, smem, sblocks, stream,
-                            w.h_ctl, w.ctl,
-                            cfg.timing ? g->gev.data() : nullptr)) {
-            for (;;) {
-                CK(cudaGraphLaunch(g->round_exec, stream));
-                launches += 2 * R;
-                search_launches += R;
-                rounds += R;
-                CK(cudaStreamSynchronize(stream));
-                graph_launches++;
-                if (cfg.timing) {
-                    for (int r = 0; r < R; r++) {
-                        float x = 0.f;
-                        CK(cudaEventElapsedTime(&x, g->gev[2 * r], g->gev[2 * r + 1]));
-                        graph_search_ms += x;
-                    }
-                }
-                if (w.h_ctl->active[(rounds - 1) & 1] == 0) break;
-                if (past_deadline()) break;
+        sw.clean = false;
+        A.words = sw.words;
+        A.slots = (StreamSlot *)sw.slots;
+        A.status = sw.status;
+        A.mask = sw.mask;
+        A.mask2 = sw.mask + sw.ring / STREAM_GS_MIN;
+        A.maps = sw.maps;
+        A.used = sw.used;
+        A.dirty = sw.dirty;
+        A.dead = sw.dead;
+        A.tasks = sw.tasks;
+        A.task_next = sw.task_links;
+        A.block_next = sw.task_links + STREAM_TASKS;
+        A.block_open = sw.task_links + 2 * STREAM_TASKS;
+        A.team_next = sw.task_links + 3 * STREAM_TASKS;
+        A.teams = sw.teams;
+        // one CUDA graph: set-up, the stream kernel, MNI, results, control words
+        int64_t n = 0;
+        auto body = [&](bool captured) {
+            const unsigned fl = captured ? cudaEventRecordExternal : cudaEventRecordDefault;
+            n = 0;
+            cudaMemsetAsync(w.ctl, 0, sizeof(Ctl), stream);
+            k_init<<<(P + 255) / 256, 256, 0, stream>>>(B);
+            if (tev) cudaEventRecordWithFlags(tev[0], stream, fl);
+            launch_stream(B, A, cfg.cyclic, stream_blocks, stream);
+            if (tev) cudaEventRecordWithFlags(tev[1], stream, fl);
+            n += 2;
+            if (B.deadline_ns) {
+                launch_stream_expire(B, A, stream);
+                n += 2;
             }
-            graph_done = true;
+            launch_mni_finalize(B, cfg, sblocks, stream, mev, fl, n);
+            cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+        };
+        if (use_graph && !capture_graph(g, &g->stream_exec, stream, [&] { body(true); })) {
+            CK(cudaGraphLaunch(g->stream_exec, stream));
+            c.graph_launches++;
         } else {
-            g->graph_fallbacks++;
+            if (use_graph) g->graph_fallbacks++;
+            body(false);
+            CK(cudaGetLastError());
         }
-    }
-    if (!graph_done) for (;;) {
-        for (int r = 0; r < R; r++) {
-            const int q = (int)(rounds & 1);
-            launch_commit(B, q, small_commit, commit_blocks, smem, stream);
-            if (cfg.timing) {
-                while (evi + 2 > g->sev.size()) {
-                    cudaEvent_t e;
-                    CK(cudaEventCreate(&e));
-                    g->sev.push_back(e);
-                }
-                CK(cudaEventRecord(g->sev[evi], stream));
-            }
-            launch_search(B, q, sblocks, stream);
-            if (cfg.timing) {
-                CK(cudaEventRecord(g->sev[evi + 1], stream));
-                evi += 2;
-            }
-            launches += 2;
-            search_launches++;
-            rounds++;
-        }
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream));
+        c.launches += n;
+        c.search_launches++;
+        c.rounds++;
+        c.reads++;
         CK(cudaStreamSynchronize(stream));
-        if (w.h_ctl->active[(rounds - 1) & 1] == 0) break;
-        if (past_deadline()) break;
+        if (tev) {
+            float x = 0.f;
+            CK(cudaEventElapsedTime(&x, tev[0], tev[1]));
+            c.search_ms += x;
+        }
+        add_mni();
+        if (!w.h_ctl->expired) sw.clean = true;
+    } else {
+        // large batches walk a list of the patterns still active; small ones launch a block per slot
+        if (P > list_threshold) B.alist = w.alist;
+        // large batches with windows of <= 1024 slots: the small-horizon commit, one full wave
+        const bool small_commit = P > list_threshold && Wmax <= SMALL_COMMIT_WMAX;
+        const int commit_blocks = small_commit ? g->commit_small_blocks : P > list_threshold ? list_threshold : P;
+        CK(cudaMemsetAsync(w.ctl, 0, sizeof(Ctl), stream));
+        k_init<<<(P + 255) / 256, 256, 0, stream>>>(B);
+        c.launches += 1;
+        rc = run_rounds(g, w, B, cfg, small_commit, commit_blocks, stream, use_graph, t_start, c);
+        if (rc) return rc;
+        launch_mni_finalize(B, cfg, sblocks, stream, mev, cudaEventRecordDefault, c.launches);
+        k_clear_used<<<(int)(((int64_t)P * 32 + 255) / 256), 256, 0, stream>>>(B);
+        c.launches += 1;
+        CK(cudaGetLastError());
     }
-    if (timed_out) {
-        k_cancel<<<(P + 255) / 256, 256, 0, stream>>>(B, nullptr, P);
-        launches += 1;
-    }
-    cudaEvent_t m0 = nullptr, m1 = nullptr;
-    if (cfg.timing) {
-        CK(cudaEventCreate(&m0));
-        CK(cudaEventCreate(&m1));
-    }
-    k_mni_setup<<<1, 1024, 0, stream>>>(B);
-    if (cfg.timing) CK(cudaEventRecord(m0, stream));
-    k_mni<<<sblocks, SEARCH_THREADS, 0, stream>>>(B);
-    if (cfg.timing) CK(cudaEventRecord(m1, stream));
-    k_finalize<<<(P + 255) / 256, 256, 0, stream>>>(B);
-    k_clear_used<<<(int)(((int64_t)P * 32 + 255) / 256), 256, 0, stream>>>(B);
-    launches += 4;
-    CK(cudaGetLastError());
-    w.clean = std::max(clean0, P);
+    w.clean = std::max(clean0, H);
     flexis_stats est{};
     if (cfg.count_maps || cfg.exact_mis) {
         const int rc2 = dev_enumerate(g, d_plans, P, d_results, stream, cfg, &est, t_start);
@@ -1346,20 +1399,21 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
     CK(cudaEventRecord(g->ev[1], stream));
     CK(cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
+    if (!streamed) add_mni();
     if (stats) {
         memset(stats, 0, sizeof *stats);
-        stats->rounds = rounds;
+        stats->rounds = c.rounds;
         stats->search_items = (int64_t)w.h_ctl->search_items;
         stats->mni_items = (int64_t)w.h_ctl->mni_items;
-        stats->kernel_launches = launches;
+        stats->kernel_launches = c.launches;
         stats->alg_bytes_greedy = (int64_t)w.h_ctl->bytes_greedy;
         stats->alg_bytes = (int64_t)(w.h_ctl->bytes_greedy + w.h_ctl->bytes_mni);
         stats->search_scanned = (int64_t)w.h_ctl->alg_scanned;
         stats->search_bound = (int64_t)w.h_ctl->alg_bound;
         stats->search_map_words = (int64_t)w.h_ctl->alg_map_words;
-        stats->search_launches = search_launches;
-        stats->graph_launches = (int32_t)graph_launches;
-        stats->d2h_bytes = (int64_t)sizeof(Ctl) * (rounds / R + 1);  // control-word reads
+        stats->search_launches = c.search_launches;
+        stats->graph_launches = (int32_t)c.graph_launches;
+        stats->d2h_bytes = (int64_t)sizeof(Ctl) * (c.reads + 1);  // control-word reads
         stats->kernel_launches += est.kernel_launches;
         stats->enum_rows = est.enum_rows;
         stats->enum_scanned = est.enum_scanned;
@@ -1367,21 +1421,9 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
         float t = 0.f;
         cudaEventElapsedTime(&t, g->ev[0], g->ev[1]);
         stats->total_ms = t;
-        if (cfg.timing) {
-            float sum = 0.f;
-            for (size_t k = 0; k < evi; k += 2) {
-                float x = 0.f;
-                cudaEventElapsedTime(&x, g->sev[k], g->sev[k + 1]);
-                sum += x;
-            }
-            stats->search_ms = sum + graph_search_ms;
-            float y = 0.f;
-            cudaEventElapsedTime(&y, m0, m1);
-            stats->mni_ms = y;
-        }
+        stats->search_ms = c.search_ms;
+        stats->mni_ms = mni_ms;
     }
-    if (m0) cudaEventDestroy(m0);
-    if (m1) cudaEventDestroy(m1);
     return FLEXIS_OK;
 }
 
@@ -1390,7 +1432,8 @@ int dev_eval_host(DeviceGraph *g, const Plan *h_plans, int32_t P, flexis_support
     if (P <= 0) return FLEXIS_OK;
     CK(cudaSetDevice(g->device));
     Workspace &w = g->ws;
-    int rc = ws_ensure(g, w, P, std::max(32, std::min(cfg.w_max, 16384)), cfg.record_selected);
+    int rc = ws_ensure(g, w, P, cfg.streamed ? 0 : P, std::max(32, std::min(cfg.w_max, 16384)),
+                       cfg.record_selected);
     if (rc) return rc;
     CK(cudaMemcpyAsync(w.plans, h_plans, sizeof(Plan) * (size_t)P, cudaMemcpyHostToDevice, g->stream));
     rc = dev_eval(g, w.plans, P, w.results, g->stream, cfg, stats);
@@ -1510,7 +1553,7 @@ int dev_support_noalloc(DeviceGraph *g, const Plan *h_plan, flexis_support_resul
     CK(cudaMemsetAsync(B.used, 0, sizeof(uint32_t) * (size_t)g->view.words, stream));
     CK(cudaMemsetAsync(B.ctl, 0, sizeof(Ctl), stream));
     k_init<<<1, 256, 0, stream>>>(B);
-    const int sblocks = g->sm_count * 6;
+    const int sblocks = g->sm_count * 4;
     Ctl h_ctl;
     for (int64_t round = 0;;) {
         for (int r = 0; r < 2; r++, round++) {
@@ -1592,7 +1635,9 @@ int serve_create(DeviceGraph *g, int32_t slots, int32_t wmin, int32_t wmax, int3
     if (wmax > 0) s->Wmax = std::max(32, std::min(wmax, 16384));
     if (wmin > 0) s->Wmin = std::max(1, std::min(wmin, s->Wmax));
     if (budget != 0) s->budget = budget;
-    int rc = ws_ensure(g, s->w, slots, s->Wmax, 0);
+    int rc = dev_edge_set(g);
+    if (rc) { delete s; return rc; }
+    rc = ws_ensure(g, s->w, slots, slots, s->Wmax, 0);
     if (rc) { serve_destroy(s); return rc; }
     if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMalloc(&s->d_admit, sizeof(int32_t) * slots) != cudaSuccess ||
