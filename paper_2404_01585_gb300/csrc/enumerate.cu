@@ -4,12 +4,12 @@
 //
 // Unlike the greedy search of kernels.cu, which stops at the first map of each root, this path
 // keeps every partial map: level i of the frontier holds rows [pattern, t_0 .. t_i] (the data
-// vertices bound to the first i+1 levels of the pattern's matching order).  One warp extends one
-// row: it finds the label slices of the row's bound neighbours of level i+1, scans the shortest
-// one 32 candidates at a time (coalesced loads), tests each candidate against the others by
-// binary search, against injectivity and against the one-hop label/degree filter, and keeps the
-// survivors (ballot).  The survivors of a chunk are staged in shared memory and written out as
-// one contiguous, coalesced block of rows.
+// vertices bound to the first i+1 levels of the pattern's matching order).  A warp extends up to 32
+// rows: every lane finds the label slices of its row's bound neighbours of level i+1, the warp scans the
+// shortest ones end to end, 32 candidates at a time, tests each against the others, against
+// injectivity and against the one-hop label/degree filter, and keeps the survivors (ballot).  The
+// survivors of a chunk are staged in shared memory and written out as one contiguous, coalesced
+// block of rows.
 //
 // The frontier of a level is capped (options.frontier_rows, at least the largest degree): a
 // count pass gives each row's survivor count, an exclusive scan gives output offsets, and the
@@ -53,6 +53,7 @@ struct EnumPass {
     unsigned long long *maps_n;             // [P] maps materialised (may pass maps_per: overflow)
     int32_t maps_per;
     unsigned long long *next;               // row counter of this launch
+    int32_t group;                          // rows a warp takes at a time (<= 32)
     unsigned long long *stat;               // [EST_N]
 };
 
@@ -104,123 +105,198 @@ __global__ void k_enum_prefix(const Plan *plans, int32_t P, unsigned long long *
     if (tid == 0) prefix[P] = carry;
 }
 
+// The rows a warp works on.
+struct EnumWarp {
+    int32_t row[32][MAXN + 1];        // pattern, t_0 .. t_i
+    uint32_t lo[32], pre[32], em[32]; // driver slice: begin, entries of the rows before; levels left to test
+    uint32_t cnt[32];                 // survivors
+    uint2 sl[32][MAXN - 1];           // the slice of every backward level (no edge set only)
+    int32_t stage[32 * (MAXN + 1)];   // a chunk's survivors on their way out
+};
+
 // Extend rows of level E.level by one level.  WRITE = false: count pass (per-row survivor counts
 // of non-final rows; last-level survivors counted into n_maps and materialised for exact MIS).
 // WRITE = true: write pass (survivors of non-final rows written at their scan offsets).
+//
+// A warp takes E.group consecutive rows: each lane finds the slices of its own row, then the lanes go over the
+// rows' candidates laid end to end, 32 at a time, each finding the row it is in by a search of the
+// rows' prefix sums.  Slices are short (six entries on average in the MiCo-shaped graph), so a row a
+// warp left most lanes idle and paid one chain of dependent loads -- plan, row, slice, candidates --
+// per row.  The rows are consecutive, so the survivors of a chunk are too: one block of the output.
 template <bool WRITE>
 __global__ void __launch_bounds__(ENUM_THREADS) k_extend(EnumPass E) {
-    __shared__ WarpState ws[ENUM_WARPS];
-    __shared__ int32_t stage[ENUM_WARPS][32 * (MAXN + 1)];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    WarpState &W = ws[wid];
-    int32_t *sg = stage[wid];
+    __shared__ EnumWarp ws[ENUM_WARPS];
+    const DevGraphView &G = E.G;
+    const int lane = threadIdx.x & 31;
+    EnumWarp &W = ws[threadIdx.x >> 5];
     const int i = E.level, j = i + 1;
     const int in_w = i + 2, out_w = i + 3;  // row widths (pattern id + vertices)
-    unsigned long long bytes = 0, scanned = 0, surv = 0, rows = 0;
-    uint32_t probes = 0;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned long long scanned = 0, surv = 0, rows = 0;
+    uint32_t probes = 0, looked = 0;  // (per lane) words read by candidate tests, slices looked up
     for (;;) {
-        unsigned long long r = 0;
-        if (lane == 0) r = atomicAdd(E.next, 1ull);
-        r = __shfl_sync(FULLMASK, r, 0);
-        if (r >= (unsigned long long)E.nrows) break;
-        if (WRITE && E.off[r + 1] == E.off[r]) continue;  // final row or no survivor
-        const long long row = E.row0 + (long long)r;
-        int p;
-        int32_t x = 0;
+        unsigned long long r0 = 0;
+        if (lane == 0) r0 = atomicAdd(E.next, (unsigned long long)E.group);
+        r0 = __shfl_sync(FULLMASK, r0, 0);
+        if (r0 >= (unsigned long long)E.nrows) break;
+        const int m = (int)min((unsigned long long)E.group, (unsigned long long)E.nrows - r0);
+        bool ok = lane < m;
+        unsigned long long wbase = 0;
+        if (WRITE) {
+            const unsigned long long o0 = E.off[r0 + min(lane, m)], o1 = E.off[r0 + min(lane + 1, m)];
+            ok = o1 != o0;  // otherwise a final row, or no survivor
+            if (!__any_sync(FULLMASK, ok)) continue;
+            wbase = __shfl_sync(FULLMASK, o0, 0) - E.off[0];
+        }
+        const long long row = E.row0 + (long long)r0;
+        __syncwarp();
         if (i == 0) {
-            // virtual row: the (row - prefix[p])-th root of pattern p
-            int lo = 0, hi = E.P;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (E.root_prefix[mid] <= (unsigned long long)row) lo = mid; else hi = mid;
+            if (ok) {
+                // virtual row: the (row - prefix[p])-th root of pattern p
+                const unsigned long long x = (unsigned long long)(row + lane);
+                int lo = 0, hi = E.P;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (E.root_prefix[mid] <= x) lo = mid; else hi = mid;
+                }
+                W.row[lane][0] = lo;
+                W.row[lane][1] = __ldg(G.lab_vtx + E.plans[lo].root_begin + (long long)(x - E.root_prefix[lo]));
             }
-            p = lo;
-            if (lane == 1) x = __ldg(E.G.lab_vtx + E.plans[p].root_begin + (row - (long long)E.root_prefix[p]));
         } else {
             const int32_t *src = E.in + row * in_w;
-            x = lane < in_w ? src[lane] : 0;
-            p = __shfl_sync(FULLMASK, x, 0);
+            for (int k = lane; k < m * in_w; k += 32) W.row[k / in_w][k % in_w] = src[k];
         }
-        const Plan &P = E.plans[p];
-        // the count pass drops rows of patterns that need nothing more; the write pass never
-        // does (the row's output slots are reserved and must hold valid rows)
-        if (!WRITE && enum_stopped(E, P, p)) {
-            if (lane == 0) E.cnt[r] = 0;
-            continue;
-        }
-        load_level_plan(W, P.greedy, P);
-        if (lane >= 1 && lane <= j) W.t[lane - 1] = x;
+        W.cnt[lane] = 0;
         __syncwarp();
-        rows++;
-        const bool final = j == P.n - 1;
-        bool ok = true;
-        if (i == 0) {
-            bytes += 32;
-            ok = vertex_fits(E.G, W.t[0], W.L.deg[0], W.need[W.L.vert[0]]);
-        }
-        uint32_t lo = 0, hi = 0;
-        if (ok) ok = enter_level(E.G, W, j, bytes, lo, hi);
-        unsigned long long total = 0;
-        unsigned long long wbase = WRITE ? E.off[r] - E.off[0] : 0;
-        if (ok) {
-            const uint4 C = W.C[j];
-            for (uint32_t pos = lo; pos < hi; pos += 32) {
-                const uint32_t k = pos + lane;
-                int32_t c = -1;
-                bool good = false;
-                uint32_t rej = 0;
-                if (k < hi) {
-                    c = __ldg(E.G.adj + k);
-                    good = check_candidate(E.G, W, C, j, c, nullptr, probes, rej);
-                }
-                const unsigned mask = __ballot_sync(FULLMASK, good);
-                scanned += min(32u, hi - pos);
-                if (!mask) continue;
-                const int nm = __popc(mask);
-                const int q = __popc(mask & ((1u << lane) - 1u));  // rank of this survivor
-                total += nm;
-                if (!WRITE && final && P.exact_mis && E.maps) {
-                    unsigned long long b0 = 0;
-                    if (lane == 0) b0 = atomicAdd(E.maps_n + p, (unsigned long long)nm);
-                    b0 = __shfl_sync(FULLMASK, b0, 0);
-                    const unsigned long long idx = b0 + q;
-                    if (good && idx < (unsigned long long)E.maps_per) {
-                        int32_t *m = E.maps + ((size_t)p * E.maps_per + idx) * MAXN;
-                        for (int l = 0; l < MAXN; l++) m[l] = l < j ? W.t[l] : (l == j ? c : -1);
+        const int p = ok ? W.row[lane][0] : -1;
+        unsigned left = __ballot_sync(FULLMASK, ok);
+        while (left) {  // the rows of one pattern (rows are ordered by pattern)
+            const int q = __shfl_sync(FULLMASK, p, __ffs(left) - 1);
+            const unsigned mine = __ballot_sync(FULLMASK, p == q);
+            left &= ~mine;
+            const Plan &P = E.plans[q];
+            // the count pass drops rows of patterns that need nothing more; the write pass never
+            // does (the row's output slots are reserved and must hold valid rows)
+            if (!WRITE && __any_sync(FULLMASK, enum_stopped(E, P, q))) continue;
+            const LevelPlan &L = P.greedy;
+            const bool last = j == P.n - 1;
+            const uint4 C = level_const(L, P.n, j, P.need[L.vert[j]]);
+            uint32_t lo = 0, len = 0, em = 0;
+            bool in = p == q;
+            if (in && i == 0) {
+                looked += 4;
+                in = vertex_fits(G, W.row[lane][1], L.deg[0], P.need[L.vert[0]]);
+            }
+            if (in) {
+                const uint32_t lab = L.lab[j], dirs = L.bdir[j];
+                uint32_t bm = L.bmask[j];
+                int db = 0;
+                len = 0xFFFFFFFFu;
+                while (bm && len) {
+                    const int b = __ffs(bm) - 1;
+                    bm &= bm - 1;
+                    const uint2 r = lane_slice(G, W.row[lane][1 + b], lab, (dirs >> (2 * b)) & 3u);
+                    looked++;
+                    if (!has_edges(G)) W.sl[lane][b] = r;
+                    if (r.y - r.x < len) {
+                        lo = r.x;
+                        len = r.y - r.x;
+                        db = b;
                     }
                 }
-                if (WRITE && !final) {
+                em = L.bmask[j] & ~(1u << db);
+            }
+            rows += __popc(mine);
+            if (!WRITE && last && !(P.exact_mis && E.maps) && !(L.bmask[j] & (L.bmask[j] - 1u))) {
+                // Counting the last level, joined to one earlier vertex: every entry of the slice completes a map
+                // but the row's own vertices (the label/degree filter rejects only vertices of no map).
+                // The entries are not read: 48 counts on 100k vertices took 87 ms with a scan of them.
+                uint32_t n = 0;
+                if (in && len) {
+                    n = len;
+                    for (uint32_t im = C.z >> 8 & 0xFFu; im; im &= im - 1)
+                        n -= contains(G.adj, lo, lo + len, W.row[lane][1 + __ffs(im) - 1], probes);
+                }
+                const unsigned long long found = warp_sum((unsigned long long)n);
+                surv += found;
+                if (found && lane == 0) atomicAdd(E.n_maps + q, found);
+                continue;
+            }
+            uint32_t x = len;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULLMASK, x, o);
+                if (lane >= o) x += y;
+            }
+            const uint32_t total = __shfl_sync(FULLMASK, x, 31);
+            __syncwarp();
+            W.lo[lane] = lo;
+            W.pre[lane] = x - len;
+            W.em[lane] = em;
+            __syncwarp();
+            scanned += total;
+            unsigned long long found = 0;
+            for (uint32_t base = 0; base < total; base += 32) {
+                const uint32_t k = base + lane;
+                int32_t c = -1;
+                int o = 0;
+                bool good = false;
+                if (k < total) {
+#pragma unroll
+                    for (int h = 16; h; h >>= 1)
+                        if (W.pre[o + h] <= k) o += h;  // the last row that begins at or before k
+                    const int32_t *t = W.row[o] + 1;
+                    c = __ldg(G.adj + W.lo[o] + (k - W.pre[o]));
+                    good = true;
+                    for (uint32_t im = C.z >> 8 & 0xFFu; im; im &= im - 1) good &= t[__ffs(im) - 1] != c;
+                    uint32_t e = W.em[o];
+                    if (good) good = admit(G, t, C, c, nullptr, has_edges(G) ? e : 0u, -1, probes);
+                    if (!has_edges(G))
+                        for (; e && good; e &= e - 1) {
+                            const uint2 r = W.sl[o][__ffs(e) - 1];
+                            good = contains(G.adj, r.x, r.y, c, probes);
+                        }
+                }
+                const unsigned mask = __ballot_sync(FULLMASK, good);
+                if (!mask) continue;
+                const int nm = __popc(mask);
+                const int rank = __popc(mask & lt);
+                found += nm;
+                if (!WRITE && !last && good) atomicAdd(&W.cnt[o], 1u);
+                if (!WRITE && last && P.exact_mis && E.maps) {
+                    unsigned long long b0 = 0;
+                    if (lane == 0) b0 = atomicAdd(E.maps_n + q, (unsigned long long)nm);
+                    const unsigned long long idx = __shfl_sync(FULLMASK, b0, 0) + rank;
+                    if (good && idx < (unsigned long long)E.maps_per) {
+                        int32_t *d = E.maps + ((size_t)q * E.maps_per + idx) * MAXN;
+                        for (int l = 0; l < MAXN; l++) d[l] = l < j ? W.row[o][1 + l] : (l == j ? c : -1);
+                    }
+                }
+                if (WRITE) {
                     // stage the chunk's rows in shared memory, then write them as one block
                     if (good) {
-                        int32_t *o = sg + q * out_w;
-                        o[0] = p;
-                        for (int l = 0; l < j; l++) o[1 + l] = W.t[l];
-                        o[1 + j] = c;
+                        int32_t *d = W.stage + rank * out_w;
+                        for (int l = 0; l <= j; l++) d[l] = W.row[o][l];
+                        d[1 + j] = c;
                     }
                     __syncwarp();
                     int32_t *dst = E.out + (size_t)wbase * out_w;
-                    for (int w = lane; w < nm * out_w; w += 32) dst[w] = sg[w];
+                    for (int w = lane; w < nm * out_w; w += 32) dst[w] = W.stage[w];
                     wbase += nm;
                     __syncwarp();
                 }
             }
+            surv += found;
+            if (!WRITE && last && found && lane == 0) atomicAdd(E.n_maps + q, found);
         }
-        surv += total;
-        if (!WRITE && lane == 0) {
-            if (final) {
-                E.cnt[r] = 0;
-                if (total) atomicAdd(E.n_maps + p, total);
-            } else {
-                E.cnt[r] = total;
-            }
-        }
+        __syncwarp();
+        if (!WRITE && lane < m) E.cnt[r0 + lane] = W.cnt[lane];
     }
-    const unsigned long long pb = warp_sum((unsigned long long)probes * 4ull);
+    const unsigned long long rb = warp_sum((unsigned long long)probes * 4ull + looked * 8ull);
     if (lane == 0 && !WRITE) {
         atomicAdd(E.stat + EST_ROWS, rows);
         atomicAdd(E.stat + EST_SCANNED, scanned);
         atomicAdd(E.stat + EST_SURVIVORS, surv);
-        atomicAdd(E.stat + EST_BYTES, bytes + pb + 4ull * scanned);
+        atomicAdd(E.stat + EST_BYTES, rb + 4ull * scanned);
     }
 }
 
@@ -726,6 +802,12 @@ struct EnumRun {
         return FLEXIS_OK;
     }
 
+    // Rows a warp takes at a time: 32, or fewer when that would leave warps without two turns.
+    int group(long long n) const {
+        const long long k = n / (2ll * blocks * ENUM_WARPS);
+        return k >= 32 ? 32 : k >= 16 ? 16 : k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1;
+    }
+
     // Process rows [0, nrows) of level `level` (level 0: virtual roots).
     int level(int lv, long long nrows) {
         const int64_t C = w->C;
@@ -738,6 +820,7 @@ struct EnumRun {
             e.row0 = a;
             e.nrows = n;
             e.cnt = w->off[lv];
+            e.group = group(n);
             CK(cudaMemsetAsync(w->ctl, 0, sizeof(unsigned long long), s));
             k_extend<false><<<blocks, ENUM_THREADS, 0, s>>>(e);
             launches++;
@@ -767,6 +850,7 @@ struct EnumRun {
                     f.in = lv > 0 ? w->rows[lv] : nullptr;
                     f.row0 = a + pos;
                     f.nrows = (long long)end - pos;
+                    f.group = group(f.nrows);
                     f.off = w->off[lv] + pos;
                     f.out = w->rows[lv + 1];
                     CK(cudaMemsetAsync(w->ctl, 0, sizeof(unsigned long long), s));
