@@ -170,7 +170,8 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
         const int bucket = tune_bucket(cnt);
         auto it = g->tuned_budget.find(bucket);
         if (it == g->tuned_budget.end()) {
-            const int32_t slice = std::max<int32_t>(512, std::min<int32_t>(cnt / 8, 8192));
+            // (the streaming greedy has no budget to choose: a token slice)
+            const int32_t slice = c2.streamed ? 32 : std::max<int32_t>(512, std::min<int32_t>(cnt / 8, 8192));
             float best_ms = 0.f;
             int32_t best = 0;
             for (int32_t cand : TUNE_CANDIDATES) {

@@ -774,6 +774,7 @@ struct Workspace {
     int64_t slots = 0;       // window-slot capacity (H x window size)
     int64_t sel_slots = 0;   // selection-log capacity (patterns x maps)
     int64_t bytes = 0;       // device bytes held
+    unsigned char *base = nullptr;  // the allocation that holds the buffers
     PatState *st = nullptr;
     uint32_t *used = nullptr;
     int32_t *dirty = nullptr;
@@ -788,7 +789,8 @@ struct Workspace {
     Plan *plans = nullptr;                   // device plan array (host-plan entry points)
     flexis_support_result *results = nullptr;
     int32_t plans_cap = 0;
-    Ctl *h_ctl = nullptr;                    // pinned
+    Ctl *h_ctl = nullptr;                    // pinned, and behind it:
+    unsigned char *h_stage = nullptr;        // [WS_STAGE] pinned, results on their way to the caller
 };
 
 // Buffers of the streaming greedy (stream.cu); all-zero claim words, status words and bitmaps
@@ -797,6 +799,7 @@ struct StreamWS {
     int32_t S = 0;           // slots
     int64_t ring = 0;        // roots in flight over all slots
     int64_t bytes = 0;
+    unsigned char *base = nullptr;  // the allocation that holds the buffers
     bool clean = false;
     unsigned long long *words = nullptr;
     void *slots = nullptr;
@@ -825,7 +828,9 @@ struct DeviceGraph {
     cudaEvent_t ev[2]{};
     std::vector<cudaEvent_t> sev;
     cudaGraphExec_t round_exec = nullptr;  // the captured round loop of the last level
-    cudaGraphExec_t stream_exec = nullptr; // the captured streaming evaluation
+    cudaGraphExec_t stream_exec = nullptr; // the captured streaming evaluation,
+    std::vector<unsigned char> stream_key; // what it was launched with,
+    int64_t stream_nodes = 0;              // its kernels
     std::vector<cudaEvent_t> gev;          // search-launch events of a group of rounds
     int64_t graph_instantiations = 0, graph_fallbacks = 0;
     int commit_small_blocks = 0;  // one wave of the small-horizon commit kernel

@@ -912,13 +912,31 @@ int dev_graph_create(const HostGraph &hg, int device, DeviceGraph **out) {
     return FLEXIS_OK;
 }
 
+// A workspace's buffers lie in one allocation: a dozen allocations each were a quarter of the first small
+// query on a new graph.
+struct Arena {
+    std::vector<std::pair<void **, size_t>> parts;
+    size_t total = 0;
+    template <class T>
+    void add(T **ptr, size_t n) {
+        parts.emplace_back(reinterpret_cast<void **>(ptr), total);
+        total += (std::max<size_t>(n * sizeof(T), 16) + 255) & ~(size_t)255;
+    }
+    int get(unsigned char **base) {
+        CK(cudaMalloc((void **)base, total));
+        for (auto &p : parts) *p.first = *base + p.second;
+        return FLEXIS_OK;
+    }
+};
+
 static void ws_free(Workspace &w) {
-    cudaFree(w.st); cudaFree(w.used); cudaFree(w.dirty); cudaFree(w.win_root); cudaFree(w.win_state);
-    cudaFree(w.win_map); cudaFree(w.items); cudaFree(w.ctl); cudaFree(w.sel_buf);
-    cudaFree(w.mni_seg); cudaFree(w.plans); cudaFree(w.results); cudaFree(w.susp); cudaFree(w.alist);
+    cudaFree(w.base);
     if (w.h_ctl) cudaFreeHost(w.h_ctl);
     w = Workspace();
 }
+
+// the pinned buffer: the control words, and results on their way to the caller
+constexpr size_t CTL_PINNED = (sizeof(Ctl) + 255) & ~(size_t)255, WS_STAGE = 64 << 10;
 
 // Capacity is kept in patterns and in window slots (patterns x Wmax) separately, so a large
 // batch with small windows followed by a small batch with large windows never allocates the
@@ -932,44 +950,41 @@ static int ws_ensure(DeviceGraph *g, Workspace &w, int32_t P, int32_t H, int32_t
     const int64_t nSel = std::max((int64_t)P * sel, w.sel_slots);
     // the captured launches hold the old buffers' addresses: they go with them
     if (&w == &g->ws) {
+        g->stream_key.clear();
         if (g->round_exec) cudaGraphExecDestroy(g->round_exec);
         g->round_exec = nullptr;
     }
     ws_free(w);
     const size_t words = (size_t)g->view.words;
-    int64_t b = 0;
-    auto alloc = [&](void **ptr, size_t bytes) {
-        b += (int64_t)bytes;
-        return cudaMalloc(ptr, std::max<size_t>(bytes, 16));
-    };
-    CK(alloc((void **)&w.st, sizeof(PatState) * nP));
-    CK(alloc((void **)&w.used, sizeof(uint32_t) * words * nH));
-    CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nH));
+    Arena a;
+    a.add(&w.st, nP);
+    a.add(&w.used, words * nH);
+    a.add(&w.dirty, (size_t)DIRTY_CAP * nH);
+    a.add(&w.win_root, (size_t)nSlots * 2);
+    a.add(&w.win_state, (size_t)nSlots * 2);
+    a.add(&w.win_map, (size_t)nSlots * 2 * MAXN);
+    a.add(&w.items, (size_t)nSlots + (size_t)nH * KSUSP);
+    a.add(&w.ctl, 1);
+    a.add(&w.mni_seg, (size_t)nP * MAXN + 1);
+    a.add(&w.susp, (size_t)nH * KSUSP * DFS_SAVE_STRIDE);
+    a.add(&w.alist, (size_t)nP * 2);
+    a.add(&w.plans, nP);
+    a.add(&w.results, nP);
+    if (nSel > 0) a.add(&w.sel_buf, (size_t)nSel * MAXN);
+    if (int rc = a.get(&w.base)) return rc;
     w.clean = 0;
-    CK(alloc((void **)&w.win_root, sizeof(int32_t) * (size_t)nSlots * 2));
-    CK(alloc((void **)&w.win_state, sizeof(int32_t) * (size_t)nSlots * 2));
-    CK(alloc((void **)&w.win_map, sizeof(int32_t) * (size_t)nSlots * 2 * MAXN));
-    CK(alloc((void **)&w.items, sizeof(int2) * ((size_t)nSlots + (size_t)nH * KSUSP)));
-    CK(alloc((void **)&w.ctl, sizeof(Ctl)));
-    CK(alloc((void **)&w.mni_seg, sizeof(unsigned long long) * ((size_t)nP * MAXN + 1)));
-    CK(alloc((void **)&w.susp, sizeof(uint32_t) * (size_t)nH * KSUSP * DFS_SAVE_STRIDE));
-    CK(alloc((void **)&w.alist, sizeof(int32_t) * (size_t)nP * 2));
-    CK(alloc((void **)&w.plans, sizeof(Plan) * (size_t)nP));
-    CK(alloc((void **)&w.results, sizeof(flexis_support_result) * (size_t)nP));
-    if (nSel > 0) CK(alloc((void **)&w.sel_buf, sizeof(int32_t) * (size_t)nSel * MAXN));
-    CK(cudaMallocHost((void **)&w.h_ctl, sizeof(Ctl)));
+    CK(cudaMallocHost((void **)&w.h_ctl, CTL_PINNED + WS_STAGE));
+    w.h_stage = reinterpret_cast<unsigned char *>(w.h_ctl) + CTL_PINNED;
     w.P = nP;
     w.H = nH;
     w.slots = nSlots;
     w.sel_slots = nSel;
-    w.bytes = b;
+    w.bytes = (int64_t)a.total;
     return FLEXIS_OK;
 }
 
 static void sws_free(StreamWS &w) {
-    cudaFree(w.words); cudaFree(w.slots); cudaFree(w.status); cudaFree(w.mask); cudaFree(w.used);
-    cudaFree(w.maps); cudaFree(w.dirty); cudaFree(w.dead);
-    cudaFree(w.tasks); cudaFree(w.task_links); cudaFree(w.teams);
+    cudaFree(w.base);
     w = StreamWS();
 }
 
@@ -980,26 +995,25 @@ static int sws_ensure(DeviceGraph *g, int32_t S, int64_t ring) {
     const int64_t nR = std::max(ring, w.ring);
     if (g->stream_exec) cudaGraphExecDestroy(g->stream_exec);
     g->stream_exec = nullptr;
+    g->stream_key.clear();
     sws_free(w);
-    int64_t b = 0;
-    auto alloc = [&](void **ptr, size_t bytes) {
-        b += (int64_t)bytes;
-        return cudaMalloc(ptr, bytes);
-    };
-    CK(alloc((void **)&w.words, sizeof(unsigned long long) * (size_t)nS));
-    CK(alloc((void **)&w.slots, sizeof(StreamSlot) * (size_t)nS));
-    CK(alloc((void **)&w.status, sizeof(uint32_t) * (size_t)(nR / STREAM_GS_MIN)));
-    CK(alloc((void **)&w.mask, sizeof(uint32_t) * (size_t)(nR / STREAM_GS_MIN) * 2));
-    CK(alloc((void **)&w.maps, sizeof(int32_t) * (size_t)nR * MAXN));
-    CK(alloc((void **)&w.used, sizeof(uint32_t) * (size_t)g->view.words * nS));
-    CK(alloc((void **)&w.dirty, sizeof(int32_t) * (size_t)DIRTY_CAP * nS));
-    CK(alloc((void **)&w.tasks, sizeof(uint32_t) * (size_t)STREAM_TASKS * STREAM_TASK_WORDS));
-    CK(alloc((void **)&w.task_links, sizeof(int32_t) * (size_t)(3 * STREAM_TASKS + STREAM_TEAMS)));
-    CK(alloc((void **)&w.teams, (size_t)STREAM_TEAMS * STREAM_TEAM_BYTES));
-    CK(alloc((void **)&w.dead, sizeof(uint32_t) * ((size_t)nS << DEAD_LOG)));
+    const size_t groups = (size_t)(nR / STREAM_GS_MIN);
+    Arena a;
+    a.add(&w.words, nS);
+    a.add(reinterpret_cast<StreamSlot **>(&w.slots), nS);
+    a.add(&w.status, groups);
+    a.add(&w.mask, groups * 2);
+    a.add(&w.maps, (size_t)nR * MAXN);
+    a.add(&w.used, (size_t)g->view.words * nS);
+    a.add(&w.dirty, (size_t)DIRTY_CAP * nS);
+    a.add(&w.tasks, (size_t)STREAM_TASKS * STREAM_TASK_WORDS);
+    a.add(&w.task_links, (size_t)(3 * STREAM_TASKS + STREAM_TEAMS));
+    a.add(&w.teams, (size_t)STREAM_TEAMS * STREAM_TEAM_BYTES);
+    a.add(&w.dead, (size_t)nS << DEAD_LOG);
+    if (int rc = a.get(&w.base)) return rc;
     w.S = nS;
     w.ring = nR;
-    w.bytes = b;
+    w.bytes = (int64_t)a.total;
     return FLEXIS_OK;
 }
 
@@ -1257,8 +1271,19 @@ static void stream_shape(const DeviceGraph *g, const EvalConfig &cfg, int32_t P,
     A.window0 = std::max(2, (S >= 128 ? 64 : 128) / A.GS);
 }
 
-int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_result *d_results,
-             cudaStream_t stream, const EvalConfig &cfg, flexis_stats *stats) {
+// What a captured streamed evaluation was launched with: an evaluation with the same bytes replays it.  (All
+// that varies between calls of one size is the contents of the buffers.)
+struct StreamKey {
+    Batch B;
+    StreamArgs A;
+    cudaStream_t stream;
+    int32_t blocks, sblocks, cyclic, mni, timed;
+};
+
+// Plans and results in host memory (h_plans, h_results; they pass through the workspace) or on the device.
+static int eval_batch(DeviceGraph *g, const Plan *h_plans, const Plan *d_plans, int32_t P,
+                      flexis_support_result *h_results, flexis_support_result *d_results, cudaStream_t stream,
+                      const EvalConfig &cfg, flexis_stats *stats) {
     if (P <= 0) return FLEXIS_OK;
     const auto t_start = std::chrono::steady_clock::now();
     CK(cudaSetDevice(g->device));
@@ -1266,16 +1291,28 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
     const int Wmin = std::max(1, std::min(cfg.w_min, Wmax));
     if (cfg.cyclic)
         if (int rc = dev_edge_set(g)) return rc;
-    const bool streamed = cfg.streamed;
-    const int32_t H = streamed ? 0 : P;  // the streaming greedy has bitmaps of its own and no windows
-    int rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected);
-    if (rc) return rc;
-    Workspace &w = g->ws;
+    bool streamed = cfg.streamed;
     StreamArgs A{};
-    int stream_blocks = 0;
+    int rc, stream_blocks = 0;
     if (streamed) {
         stream_shape(g, cfg, P, A, stream_blocks);
-        if ((rc = sws_ensure(g, A.S, (int64_t)A.S * A.RG * A.GS))) return rc;
+        // no room for its buffers: the windowed rounds, which need less for a small batch
+        rc = sws_ensure(g, A.S, (int64_t)A.S * A.RG * A.GS);
+        if (rc == FLEXIS_E_NOMEM) {
+            (void)cudaGetLastError();
+            sws_free(g->sws);
+            streamed = false;
+        } else if (rc) {
+            return rc;
+        }
+    }
+    const int32_t H = streamed ? 0 : P;  // the streaming greedy has bitmaps of its own and no windows
+    if ((rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected))) return rc;
+    Workspace &w = g->ws;
+    if (h_plans) {
+        CK(cudaMemcpyAsync(w.plans, h_plans, sizeof(Plan) * (size_t)P, cudaMemcpyHostToDevice, stream));
+        d_plans = w.plans;
+        d_results = w.results;
     }
     StreamWS &sw = g->sws;
     g->last_P = P;
@@ -1352,28 +1389,43 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
                 n += 2;
             }
             launch_mni_finalize(B, cfg, sblocks, stream, mev, fl, n);
-            cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
         };
-        if (use_graph && !capture_graph(g, &g->stream_exec, stream, [&] { body(true); })) {
+        bool replay = false;
+        if (use_graph) {
+            StreamKey k;
+            memset((void *)&k, 0, sizeof k);
+            k.B = B;
+            k.A = A;
+            k.stream = stream;
+            k.blocks = stream_blocks;
+            k.sblocks = sblocks;
+            k.cyclic = cfg.cyclic;
+            k.mni = cfg.want_mni;
+            k.timed = tev != nullptr;
+            const unsigned char *kb = reinterpret_cast<const unsigned char *>(&k);
+            replay = g->stream_exec && g->stream_key.size() == sizeof k && !memcmp(g->stream_key.data(), kb, sizeof k);
+            if (!replay) {
+                g->stream_key.clear();
+                replay = !capture_graph(g, &g->stream_exec, stream, [&] { body(true); });
+                if (replay) {
+                    g->stream_key.assign(kb, kb + sizeof k);
+                    g->stream_nodes = n;
+                } else {
+                    g->graph_fallbacks++;
+                }
+            }
+        }
+        if (replay) {
             CK(cudaGraphLaunch(g->stream_exec, stream));
             c.graph_launches++;
+            n = g->stream_nodes;
         } else {
-            if (use_graph) g->graph_fallbacks++;
             body(false);
             CK(cudaGetLastError());
         }
         c.launches += n;
         c.search_launches++;
         c.rounds++;
-        c.reads++;
-        CK(cudaStreamSynchronize(stream));
-        if (tev) {
-            float x = 0.f;
-            CK(cudaEventElapsedTime(&x, tev[0], tev[1]));
-            c.search_ms += x;
-        }
-        add_mni();
-        if (!w.h_ctl->expired) sw.clean = true;
     } else {
         // large batches walk a list of the patterns still active; small ones launch a block per slot
         if (P > list_threshold) B.alist = w.alist;
@@ -1398,8 +1450,21 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
     }
     CK(cudaEventRecord(g->ev[1], stream));
     CK(cudaMemcpyAsync(w.h_ctl, w.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream));
+    const size_t rbytes = sizeof(flexis_support_result) * (size_t)P;
+    const bool staged = h_results && rbytes <= WS_STAGE;
+    if (h_results)
+        CK(cudaMemcpyAsync(staged ? (void *)w.h_stage : (void *)h_results, d_results, rbytes, cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
-    if (!streamed) add_mni();
+    if (staged) memcpy(h_results, w.h_stage, rbytes);
+    if (streamed) {
+        if (tev) {
+            float x = 0.f;
+            CK(cudaEventElapsedTime(&x, tev[0], tev[1]));
+            c.search_ms += x;
+        }
+        if (!w.h_ctl->expired) sw.clean = true;
+    }
+    add_mni();
     if (stats) {
         memset(stats, 0, sizeof *stats);
         stats->rounds = c.rounds;
@@ -1427,20 +1492,16 @@ int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_resu
     return FLEXIS_OK;
 }
 
+int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_result *d_results,
+             cudaStream_t stream, const EvalConfig &cfg, flexis_stats *stats) {
+    return eval_batch(g, nullptr, d_plans, P, nullptr, d_results, stream, cfg, stats);
+}
+
 int dev_eval_host(DeviceGraph *g, const Plan *h_plans, int32_t P, flexis_support_result *h_results,
                   const EvalConfig &cfg, flexis_stats *stats) {
     if (P <= 0) return FLEXIS_OK;
-    CK(cudaSetDevice(g->device));
-    Workspace &w = g->ws;
-    int rc = ws_ensure(g, w, P, cfg.streamed ? 0 : P, std::max(32, std::min(cfg.w_max, 16384)),
-                       cfg.record_selected);
+    const int rc = eval_batch(g, h_plans, nullptr, P, h_results, nullptr, g->stream, cfg, stats);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(w.plans, h_plans, sizeof(Plan) * (size_t)P, cudaMemcpyHostToDevice, g->stream));
-    rc = dev_eval(g, w.plans, P, w.results, g->stream, cfg, stats);
-    if (rc) return rc;
-    CK(cudaMemcpyAsync(h_results, w.results, sizeof(flexis_support_result) * (size_t)P,
-                       cudaMemcpyDeviceToHost, g->stream));
-    CK(cudaStreamSynchronize(g->stream));
     if (stats) {
         stats->h2d_bytes += (int64_t)sizeof(Plan) * P;
         stats->d2h_bytes += (int64_t)sizeof(flexis_support_result) * P;

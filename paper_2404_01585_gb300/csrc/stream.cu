@@ -889,7 +889,13 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             g = tk >= 0 ? 0 : claim(A, s);
             if (g < 0) {
                 // (the batch's state is one line that every warp looks at: as seldom as possible)
-                if (home < 0 || (idle & 7) == 7) {
+                // (a home warp whose slot has no more patterns looks each time)
+                bool look = home < 0 || (idle & 7) == 7;
+                if (!look) {
+                    if (lane == 0) look = word_of(A.words + s) == 0ull;
+                    look = __any_sync(FULLMASK, look);
+                }
+                if (look) {
                     const int t = find_slot(A, s);
                     if (t >= 0) {
                         s = t;
@@ -907,7 +913,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                     if (++idle > IDLE_POLLS) break;
                     if (home >= 0) s = home;
                     __nanosleep(nap);
-                    nap = min(2 * nap, home >= 0 ? STREAM_NAP_HOME : STREAM_NAP_MAX);
+                    nap = min(nap + nap / 2, home >= 0 ? STREAM_NAP_HOME : STREAM_NAP_MAX);
                     continue;
                 }
             }
