@@ -105,7 +105,9 @@ static_assert(sizeof(StreamTeam) <= STREAM_TEAM_BYTES, "team record");
 // a task: the saved search state, then
 constexpr int TASK_TEAM = DFS_SAVE_WORDS, TASK_KEY = DFS_SAVE_WORDS + 1, TASK_SHIFT = DFS_SAVE_WORDS + 3;
 static_assert(TASK_SHIFT < STREAM_TASK_WORDS, "task record");
-constexpr int KEY_BITS = 48, KEY_CUT = 4;  // a cut divides a key interval by 16
+// A cut divides a key interval by 16.  After twelve of them a task that is cut again starts a team of its own:
+// where it was left uncut, one task of a six-cycle on 1M vertices ran 190 ms by itself.
+constexpr int KEY_BITS = 48, KEY_CUT = 4;
 constexpr int TASK_CUT = 1 << KEY_CUT;     // tasks of one block
 constexpr int SHIFT_ROOT = 0xFF;           // in TASK_SHIFT: the task is a root of a group, its number the key
 
@@ -1108,7 +1110,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             shift = KEY_BITS;
         }
         if (from > 0) state_of_map(G, X.W, from, bytes, probes);
-        bool shared = false;
+        bool shared = false, nested = false;  // cut; into a team below this task
         for (bool again = from > 0 || mode == M_TASK;; again = true) {
             why = STOP_NO;
             res = dfs_run<StreamStop, true>(G, X.W, A.used + (size_t)s * G.words, root, bytes, probes, steps, again,
@@ -1116,9 +1118,27 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                                                              key, B.ctl, B.deadline_ns, steps + STOP_EVERY, split_at, &why},
                                             fs, A.dead + ((size_t)s << DEAD_LOG));
             if (res != DFS_SUSPENDED || why != STOP_SPLIT) break;
-            shared = cut_search(B, A, X, mode == M_TASK ? team : -1, key, shift, mode, s, p, g, i, todo,
-                                mode == M_ROOT ? (uint32_t)gteam : found, mode == M_ROOT ? (uint32_t)task : found2, gsteps);
+            // what to go on with when a new team has decided it; a task whose key cannot be divided any more
+            // gets a team of its own
+            int tm = -1, back_i = i;
+            uint32_t back[4] = {todo, found, found2, gsteps};
+            if (mode == M_ROOT) {
+                back[1] = (uint32_t)gteam;
+                back[2] = (uint32_t)task;
+            } else if (mode == M_TASK && shift >= KEY_CUT) {
+                tm = team;
+            } else if (mode == M_TASK) {
+                nested = true;
+                back_i = shift;
+                back[0] = (uint32_t)key;
+                back[1] = (uint32_t)team;
+                back[2] = (uint32_t)task;
+                back[3] = (uint32_t)(key >> 32);
+            }
+            shared = cut_search(B, A, X, tm, nested ? 0ull : key, nested ? KEY_BITS : shift, mode, s, p, g, back_i, back[0],
+                                back[1], back[2], back[3]);
             if (shared) break;
+            nested = false;
             split_at = steps + SPLIT_AGAIN;
         }
         if (lane == 0) {
@@ -1132,9 +1152,10 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             if (mode != M_TASK) *reinterpret_cast<volatile uint32_t *>(&A.slots[s].last_steps) = steps;
         }
         __syncwarp();
-        if (shared || mode == M_TASK) {
+        bool parked = false;  // the search goes on elsewhere
+        while (shared || mode == M_TASK) {
             bool last = false;
-            if (mode == M_TASK) {
+            if (mode == M_TASK && !nested) {
                 // the task is finished, or has been replaced by its own tasks
                 StreamTeam *T = team_of(A, team);
                 if (!shared && res == DFS_FOUND && lane < MAXN)
@@ -1157,8 +1178,8 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                 last = __any_sync(FULLMASK, last);
             }
             if (!last) {
-                mode = M_CLAIM;
-                continue;
+                parked = true;
+                break;
             }
             // the shared search is decided: go on with what it belongs to
             __threadfence();
@@ -1198,6 +1219,17 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             __syncwarp();
             if (lane == 0) stack_push(&B.ctl->teams_free, A.team_next, team);
             __syncwarp();
+            shared = nested = false;
+            if (mode == M_TASK) {
+                team = (int)found;
+                task = (int)found2;
+                key = (unsigned long long)gsteps << 32 | todo;
+                shift = i;
+            }
+        }
+        if (parked) {
+            mode = M_CLAIM;
+            continue;
         }
         if (mode == M_RETIRE) continue;
         if (mode == M_ROOT) {
