@@ -518,14 +518,15 @@ int flexis_support_plans_device(flexis_graph *g, const flexis_plan *d_plans, int
     EvalConfig cfg = config_for(g, count);
     cudaStream_t s = stream ? (cudaStream_t)stream : dev_graph_stream(g->dg);
     if (count > 0) {
-        // the plans' mode flags decide which enumerator passes run: read them back (1 KB each)
+        // the plans' mode flags decide which enumerator passes run: read them back
         std::vector<Plan> h((size_t)count);
-        if (cudaMemcpyAsync(h.data(), d_plans, sizeof(Plan) * (size_t)count, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpy2DAsync(h.data(), sizeof(Plan), d_plans, sizeof(flexis_plan), sizeof(Plan), (size_t)count,
+                              cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
             return FLEXIS_E_CUDA;
         enum_config(g, h.data(), count, cfg);
     }
-    return dev_eval(g->dg, reinterpret_cast<const Plan *>(d_plans), count, d_results, s, cfg, &g->last);
+    return dev_eval(g->dg, d_plans, count, d_results, s, cfg, &g->last);
 }
 
 int flexis_last_stats(const flexis_graph *g, flexis_stats *out) {

@@ -51,7 +51,7 @@ cudaStream_t dev_graph_stream(const DeviceGraph *g);
 
 // Evaluate P compiled plans that are already in device memory; results to device memory.
 // Synchronises `stream` before returning.  stats (nullable) receives counters.
-int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_result *d_results,
+int dev_eval(DeviceGraph *g, const flexis_plan *d_plans, int32_t P, flexis_support_result *d_results,
              cudaStream_t stream, const EvalConfig &cfg, flexis_stats *stats);
 
 // Host-buffer convenience: copy plans in, evaluate, copy results out (on the graph's stream).

@@ -1280,8 +1280,9 @@ struct StreamKey {
     int32_t blocks, sblocks, cyclic, mni, timed;
 };
 
-// Plans and results in host memory (h_plans, h_results; they pass through the workspace) or on the device.
-static int eval_batch(DeviceGraph *g, const Plan *h_plans, const Plan *d_plans, int32_t P,
+// Plans and results in host memory (h_plans, h_results) or on the device (rows, d_results).  The kernels
+// read the plans in the workspace.
+static int eval_batch(DeviceGraph *g, const Plan *h_plans, const flexis_plan *rows, int32_t P,
                       flexis_support_result *h_results, flexis_support_result *d_results, cudaStream_t stream,
                       const EvalConfig &cfg, flexis_stats *stats) {
     if (P <= 0) return FLEXIS_OK;
@@ -1309,10 +1310,13 @@ static int eval_batch(DeviceGraph *g, const Plan *h_plans, const Plan *d_plans, 
     const int32_t H = streamed ? 0 : P;  // the streaming greedy has bitmaps of its own and no windows
     if ((rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected))) return rc;
     Workspace &w = g->ws;
+    const Plan *d_plans = w.plans;
     if (h_plans) {
         CK(cudaMemcpyAsync(w.plans, h_plans, sizeof(Plan) * (size_t)P, cudaMemcpyHostToDevice, stream));
-        d_plans = w.plans;
         d_results = w.results;
+    } else {  // (the caller's records are padded)
+        CK(cudaMemcpy2DAsync(w.plans, sizeof(Plan), rows, sizeof(flexis_plan), sizeof(Plan), (size_t)P,
+                             cudaMemcpyDeviceToDevice, stream));
     }
     StreamWS &sw = g->sws;
     g->last_P = P;
@@ -1492,9 +1496,9 @@ static int eval_batch(DeviceGraph *g, const Plan *h_plans, const Plan *d_plans, 
     return FLEXIS_OK;
 }
 
-int dev_eval(DeviceGraph *g, const Plan *d_plans, int32_t P, flexis_support_result *d_results,
+int dev_eval(DeviceGraph *g, const flexis_plan *rows, int32_t P, flexis_support_result *d_results,
              cudaStream_t stream, const EvalConfig &cfg, flexis_stats *stats) {
-    return eval_batch(g, nullptr, d_plans, P, nullptr, d_results, stream, cfg, stats);
+    return eval_batch(g, nullptr, rows, P, nullptr, d_results, stream, cfg, stats);
 }
 
 int dev_eval_host(DeviceGraph *g, const Plan *h_plans, int32_t P, flexis_support_result *h_results,
