@@ -1,0 +1,102 @@
+"""The streaming greedy and the enumerator at the edges of their work split: group, ring and slot
+remainders, more patterns than slots, shared searches, the edge set and the counted last level.  All
+quantities are integers: equality is exact."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import oracle
+import paper_2404_01585_gb300 as fx
+from workloads import make_graph, random_patterns
+
+pytestmark = pytest.mark.gpu
+EARLY, FULL = fx.FLEXIS_MODE_EARLY, fx.FLEXIS_MODE_FULL
+COUNT, NO_MIS = fx.FLEXIS_MODE_COUNT_MAPS, fx.FLEXIS_MODE_NO_MIS
+ALL_SHAPES = ["tree", "cycle", "clique", "path", "star"]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def key(r):
+    return (r["status"], r["tau"], r["mis"], r["mni"], bool(r["frequent"]))
+
+
+def er(nv, ne, nl, seed):
+    return make_graph(kind="er", nv=nv, ne=ne, nl=nl, law="uniform", zipf_s=None, gamma=None, seed=seed)
+
+
+# one label: every vertex is a root; a batch of 1 has groups of 8 roots, of 700 of 8 or 16, of 3000 of 32
+@pytest.mark.parametrize("count", [1, 700, 3000])
+@pytest.mark.parametrize("nv", [7, 33, 1025])
+def test_streamed_equals_windowed_and_oracle(nv, count):
+    lab, src, dst = er(nv, 3 * nv, 1, nv)
+    pats = random_patterns(count, range(2, 7), ALL_SHAPES, lab, 3)
+    g = fx.Graph(lab, src, dst)
+    w = fx.Graph(lab, src, dst, window_min=16, window_max=256)
+    for mode in (EARLY, FULL):
+        got = [key(r) for r in g.support_batch(pats, 4, 0.5, mode)]
+        assert got == [key(r) for r in w.support_batch(pats, 4, 0.5, mode)]
+    og = oracle.Graph(lab, src, dst)
+    for (pl, pe), k in list(zip(pats, got))[:6]:
+        o = og.support(pl, pe, sigma=4, lam=0.5, mode="full", tier=1)
+        assert k == (0, o["tau"], o["mis"], o["mni"], o["frequent"])
+    g.close()
+    w.close()
+
+
+@pytest.mark.parametrize("record", [1, 5000])
+def test_selection_log_of_streamed_rounds(record):
+    lab, src, dst = er(2000, 9000, 2, 8)
+    g = fx.Graph(lab, src, dst, record_selected=record)
+    w = fx.Graph(lab, src, dst, record_selected=record, window_min=16, window_max=256)
+    pats = random_patterns(9, range(2, 6), ALL_SHAPES, lab, 4)
+    a, b = (x.support_batch(pats, 3, 0.5, FULL) for x in (g, w))
+    for i in range(len(pats)):
+        assert key(a[i]) == key(b[i])
+        assert g.selected_maps(i, len(pats[i][0])) == w.selected_maps(i, len(pats[i][0])), i
+    g.close()
+    w.close()
+
+
+# few patterns whose roots need long searches: they are cut into tasks, and cut again
+@pytest.mark.parametrize("n", [5, 6, 7])
+def test_shared_searches(n):
+    lab, src, dst = make_graph(kind="cl", nv=60000, ne=240000, nl=3, law="zipf", zipf_s=1.0, gamma=2.3, seed=12)
+    cyc = np.array([[i, (i + 1) % n] for i in range(n)], np.int32)
+    pats = [(np.array([(i * k) % 3 for i in range(n)], np.int32), cyc) for k in (0, 1, 2)]
+    g = fx.Graph(lab, src, dst)
+    w = fx.Graph(lab, src, dst, window_min=16, window_max=4096)
+    for sigma in (50, 1000):
+        a, b = (x.support_batch(pats, sigma, 0.5, EARLY) for x in (g, w))
+        assert [key(r) for r in a] == [key(r) for r in b]
+    g.close()
+    w.close()
+
+
+# a warp of the enumerator takes 1 .. 32 rows; frontier_rows cuts the frontier in the middle of a group
+@pytest.mark.parametrize("nv,rows", [(2, 0), (31, 0), (33, 64), (1000, 100), (70000, 5000), (70000, 0)])
+def test_counts_in_closed_form(nv, rows):
+    rng = np.random.default_rng(nv)
+    m = min(4 * nv, nv * (nv - 1) // 2)
+    e = np.unique(np.sort(rng.integers(0, nv, (m, 2)), axis=1), axis=0)
+    hub = np.stack([np.zeros(nv - 1, np.int64), np.arange(1, nv)], 1)[: 3000]  # one long slice
+    e = np.unique(np.concatenate([e[e[:, 0] != e[:, 1]], hub]), axis=0)
+    g = fx.Graph(np.zeros(nv, np.int32), e[:, 0], e[:, 1], frontier_rows=rows)
+    A = sp.csr_matrix((np.ones(len(e)), (e[:, 0], e[:, 1])), shape=(nv, nv), dtype=np.int64)
+    A = A + A.T
+    d = np.asarray(A.sum(1)).ravel()
+    tri = int((A @ A).multiply(A).sum())  # closed walks of three steps: six a triangle
+    s = lambda *x: np.zeros(x[0], np.int32)
+    pats = [(s(2), [(0, 1)]), (s(3), [(0, 1), (0, 2)]), (s(4), [(0, 1), (0, 2), (0, 3)]),
+            (s(4), [(0, 1), (1, 2), (2, 3)]), (s(3), [(0, 1), (1, 2), (2, 0)])]
+    want = [int(d.sum()), int((d * (d - 1)).sum()), int((d * (d - 1) * (d - 2)).sum()),
+            int(((d[e[:, 0]] - 1) * (d[e[:, 1]] - 1)).sum() * 2 - tri), tri]
+    res = g.support_batch([(pl, np.array(pe, np.int32)) for pl, pe in pats], 1, 0.5, FULL | COUNT | NO_MIS)
+    assert [r["n_maps"] for r in res] == [min(x, 1 << 32) for x in want]  # counts saturate at maps_cap
+    g.close()
