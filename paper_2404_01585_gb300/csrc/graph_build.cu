@@ -257,15 +257,29 @@ __global__ void __launch_bounds__(GB_THREADS) k_slice_table(const VRec *vrec, co
     }
 }
 
+// Whether an optional table may take `bytes`: an eighth of the free memory.  (Asking costs up to a
+// millisecond; tables that no graph of use would miss room for are not worth it.)
+static bool spare(int64_t bytes) {
+    if (bytes <= (32ll << 20)) return true;
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return bytes <= (int64_t)(fr / 8);
+}
+
 int dev_slice_table(DeviceGraph *g, int nl) {
     const long long rows = g->vrec_count;
     const int64_t bytes = 4ll * rows * (nl + 1);
-    size_t fr = 0, tot = 0;
-    CK(cudaMemGetInfo(&fr, &tot));
     g->view.off = nullptr;
     g->view.nl1 = nl + 1;
-    if (nl < 1 || g->view.nv < 1 || bytes > SLICE_TABLE_BYTES || bytes > (int64_t)(fr / 8)) return FLEXIS_OK;
-    CK(cudaMalloc(&g->d_off, (size_t)bytes));
+    if (nl < 1 || g->view.nv < 1 || bytes > SLICE_TABLE_BYTES || !spare(bytes)) return FLEXIS_OK;
+    if (cudaMalloc(&g->d_off, (size_t)bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        g->d_off = nullptr;
+        return FLEXIS_OK;
+    }
     g->bytes += bytes;
     const long long want = (rows * 32 + GB_THREADS - 1) / GB_THREADS;
     const int blocks = (int)std::min<long long>(want, (long long)std::max(1, g->sm_count) * 8);
@@ -286,7 +300,9 @@ static int bit_width(unsigned long long x) {
     return b;
 }
 
-// Edge set: a warp per row inserts the row's neighbours with a larger id.
+// Edge set: a warp per row inserts the edges of which the row's vertex is the end of smaller degree (by id
+// on a tie).  Hub rows insert next to nothing that way; inserted from the end of smaller id, a row of
+// 10k neighbours kept one warp busy for 1.1 ms on the MiCo-shaped graph.
 __global__ void __launch_bounds__(GB_THREADS) k_edge_set(DevGraphView G, uint32_t *table, unsigned int *failed) {
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -294,7 +310,8 @@ __global__ void __launch_bounds__(GB_THREADS) k_edge_set(DevGraphView G, uint32_
         const uint4 r = __ldg(reinterpret_cast<const uint4 *>(G.vrec + v));
         for (uint32_t k = lane; k < r.z; k += 32) {
             const int32_t w = __ldg(G.adj + r.x + k);
-            if ((long long)w <= v) continue;
+            const uint32_t dw = __ldg(&G.vrec[w].deg);
+            if (dw < r.z || (dw == r.z && (long long)w <= v)) continue;
             uint32_t bucket, entry;
             edge_key(G, (uint32_t)v, (uint32_t)w, bucket, entry);
             bool placed = false;
@@ -317,29 +334,25 @@ int dev_edge_set(DeviceGraph *g) {
     // three edges a bucket on average: one in 80 buckets is full
     while ((3ll << V.eb_log) < g->n_arcs / 2) V.eb_log++;
     const int64_t bytes = 4ll * EDGE_WAYS << V.eb_log;
-    size_t fr = 0, tot = 0;
-    CK(cudaMemGetInfo(&fr, &tot));
-    if (bytes > EDGE_SET_BYTES || bytes > (int64_t)(fr / 8) || V.eb_log >= 32) return FLEXIS_OK;
+    if (bytes > EDGE_SET_BYTES || !spare(bytes) || V.eb_log >= 32) return FLEXIS_OK;
     V.eb_mask = (uint32_t)((1ull << V.eb_log) - 1);
-    unsigned int *failed = nullptr, h = 0;
-    CK(cudaMalloc((void **)&failed, sizeof *failed));
+    unsigned int h = 0;
     auto done = [&](int rc) {
-        cudaFree(failed);
         if (rc || h) {
             cudaFree(g->d_edges);
             g->d_edges = nullptr;
         }
         return rc;
     };
-    if (cudaMalloc(&g->d_edges, (size_t)bytes) != cudaSuccess) {
+    if (cudaMalloc(&g->d_edges, (size_t)bytes + sizeof h) != cudaSuccess) {
         (void)cudaGetLastError();
         g->d_edges = nullptr;
         return done(FLEXIS_OK);
     }
     const int blocks = (int)std::min<long long>((V.nv * 32 + GB_THREADS - 1) / GB_THREADS,
                                                 (long long)std::max(1, g->sm_count) * 8);
-    if (cudaMemsetAsync(g->d_edges, 0, (size_t)bytes, g->stream) != cudaSuccess ||
-        cudaMemsetAsync(failed, 0, sizeof *failed, g->stream) != cudaSuccess)
+    unsigned int *failed = (unsigned int *)((unsigned char *)g->d_edges + bytes);
+    if (cudaMemsetAsync(g->d_edges, 0, (size_t)bytes + sizeof h, g->stream) != cudaSuccess)
         return done(FLEXIS_E_CUDA);
     k_edge_set<<<blocks, GB_THREADS, 0, g->stream>>>(V, (uint32_t *)g->d_edges, failed);
     if (cudaGetLastError() != cudaSuccess ||
