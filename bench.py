@@ -249,7 +249,7 @@ def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2404_01585_gb300", "csrc")
-    for f in ("kernels.cu", "fx_kern.cuh", "fx.h"):
+    for f in ("stream.cu", "fx_stream.h", "fx_batch.cuh", "fx_kern.cuh", "fx.h"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -259,7 +259,7 @@ def committed_traffic(alg_bytes_per_launch):
     """DRAM bytes per launch of the search kernel, from the committed ncu capture of a small case
     (DRAM bytes per algorithmic byte there, times this run's algorithmic bytes per launch), if
     the capture was taken on the current kernel source; else None."""
-    path = os.path.join(ROOT, "profiles", "k_search_traffic.json")
+    path = os.path.join(ROOT, "profiles", "k_stream_traffic.json")
     try:
         with open(path) as f:
             d = json.load(f)
@@ -457,7 +457,7 @@ def main():
     traffic, tinfo = committed_traffic(alg_b / launches)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": "k_search (greedy root search)", "peak_kind": peak_kind,
+                "kernel": "k_stream (streaming greedy)", "peak_kind": peak_kind,
                 "alg_bytes_per_launch": alg_b / launches, "launches": launches,
                 "avg_launch_ms": stats["search_ms"] / launches,
                 "alg_terms": {"slice_entries_scanned": int(stats["search_scanned"]),

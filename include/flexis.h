@@ -101,7 +101,9 @@ typedef struct flexis_server flexis_server;
 typedef struct {
     uint64_t seed;        /* greedy-order seed (default 0x5EED) */
     int32_t device;       /* CUDA device ordinal (default 0) */
-    int32_t window_min;   /* speculation window per pattern: 0 = autotuned */
+    int32_t window_min;   /* speculation window per pattern: 0 = autotuned.  Setting this or one of
+                             window_max, search_budget, split_pieces and sub_searches runs the
+                             greedy phase in windowed rounds instead of one streaming launch */
     int32_t window_max;   /* 0 = autotuned */
     int32_t search_blocks;/* blocks of the search kernel: 0 = autotuned (multiple of the SM count) */
     int32_t record_selected; /* >0: keep up to this many selected maps per pattern (tests) */
@@ -113,16 +115,16 @@ typedef struct {
                                 0 = default, -1 = never split */
     int32_t sub_searches;    /* saved sub-searches a pattern may hold at once (1..32): 0 = default */
     int32_t timing;          /* 1: CUDA events around every search launch (stats.search_ms) */
-    int32_t graphs;          /* 0 = default (the round loop of each level is captured once into a
-                                CUDA graph and replayed), -1 = launch kernel by kernel */
+    int32_t graphs;          /* 0 = default (an evaluation's launches, or its round loop, are captured
+                                into a CUDA graph and replayed), -1 = launch kernel by kernel */
     int32_t deadline_ms;     /* > 0: wall-clock limit of one evaluation call (support, batch, each
                                 device batch of a mining level) and of one served request (from
                                 its submission).  Patterns still undecided when it passes stop
-                                between two rounds and report status FLEXIS_E_TIMEOUT, with mis =
+                                (between two rounds, or within a search) and report status FLEXIS_E_TIMEOUT, with mis =
                                 the maps committed so far (a lower bound of their mIS), mni = -1
                                 and frequent = 0 (undecided); flexis_mine then fails with
                                 FLEXIS_E_TIMEOUT.  The limit is checked between rounds of the
-                                greedy phase, and by the MNI kernel itself (device clock) every
+                                greedy phase or every 32 chunks of a streamed search, and by the MNI kernel itself (device clock) every
                                 few thousand candidate chunks of a search: a pattern whose MNI
                                 count is cut reports FLEXIS_E_TIMEOUT with its final mis and
                                 frequent and mni = -1.  0 = no limit (default). */
