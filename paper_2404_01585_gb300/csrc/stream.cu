@@ -55,8 +55,9 @@ constexpr uint32_t G_STEPS_MAX = (1u << 24) - 1;
 enum : int { STOP_NO = 0, STOP_ABORT = 1, STOP_SPLIT = 2 };
 constexpr uint32_t STOP_EVERY = 32;     // chunks between looks at the slot's state
 constexpr int IDLE_POLLS = 1 << 17;     // looks for work before an idle warp leaves
-constexpr uint32_t LANE_STEPS = 96;     // iterations of a lane's search
-constexpr uint32_t LANE_FEW_STEPS = 24, LANE_FEW = 3;  // ... once so few lanes are left
+// Iterations of a lane's search.  (MiCo-shaped mining to 5 edges: 580 ms; 640 when the last three lanes were
+// given up after 24 iterations, 600 after 48; 675 with 256 iterations.)
+constexpr uint32_t LANE_STEPS = 96;
 constexpr uint32_t STREAM_REDO_STEPS = 6;  // set-up of a second search, in chunks
 constexpr uint32_t SPLIT_STEPS = 128;   // chunks of a search before it is shared with idle warps
 constexpr uint32_t SPLIT_AGAIN = 4096;  // ... before the next try, after one that failed
@@ -400,8 +401,8 @@ __device__ __forceinline__ void retire_begin(const StreamArgs &A, StreamWarp &X,
 
 // A lane searches its own root (plain backtracking, one candidate an iteration) while the others search
 // theirs: 32 roots for the dependent accesses of one.  Most roots of most patterns are decided within
-// a few candidates a level; the ones that are not when only a few lanes are left, or after
-// LANE_STEPS iterations, are left to the whole warp (`open`).  Maps go to X.gm; returns the lanes that
+// a few candidates a level; the ones that are not after LANE_STEPS iterations are left to the whole
+// warp (`open`).  Maps go to X.gm; returns the lanes that
 // found one.  The per-level positions share W.sl with the warp's searches.
 template <class View>
 __device__ __forceinline__ uint32_t lane_searches(const View &G, StreamWarp &X, const uint32_t *used,
@@ -420,8 +421,7 @@ __device__ __forceinline__ uint32_t lane_searches(const View &G, StreamWarp &X, 
     if (ok) t[0] = root;
     uint32_t it = 0;
     for (;; it++) {
-        const uint32_t left = __popc(__ballot_sync(FULLMASK, act));
-        if (left == 0 || it >= LANE_STEPS || (it >= LANE_FEW_STEPS && left <= LANE_FEW)) break;
+        if (it >= LANE_STEPS || !__any_sync(FULLMASK, act)) break;
         if (!act) continue;
         if (pos >= hi) {
             // level i is exhausted: when nothing but the vertex at level i - 1 had a part in that, it is
