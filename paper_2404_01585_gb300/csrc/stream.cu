@@ -1092,6 +1092,9 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                 if (lane == 0) end = *reinterpret_cast<volatile int32_t *>(&B.ctl->expired);
                 if (__any_sync(FULLMASK, end)) break;
             }
+            // Whoever ends the pattern clears what this warp wrote for it (dead candidates, maps): every lane's
+            // stores come before the reference falls.  An aborted search gets here with no fence of its own.
+            __threadfence();
             __syncwarp();
             unsigned long long w = 0;
             if (lane == 0) w = atomicAdd(A.words + s, 0ull - W_REF1);

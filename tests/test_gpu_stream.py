@@ -100,3 +100,21 @@ def test_counts_in_closed_form(nv, rows):
     res = g.support_batch([(pl, np.array(pe, np.int32)) for pl, pe in pats], 1, 0.5, FULL | COUNT | NO_MIS)
     assert [r["n_maps"] for r in res] == [min(x, 1 << 32) for x in want]  # counts saturate at maps_cap
     g.close()
+
+
+# Few slots and caps of one to a few maps: a pattern that reaches its cap aborts the searches ahead of it, and
+# its slot goes to the next pattern at once.  What the aborted searches knew of the old pattern must not
+# reach the new one; the patterns share labels, so that an old dead candidate would be one of the new.
+@pytest.mark.parametrize("blocks", [1, 2])
+@pytest.mark.parametrize("sigma", [1, 40])
+def test_slots_reused_after_aborted_searches(blocks, sigma):
+    lab, src, dst = make_graph(kind="cl", nv=20000, ne=120000, nl=2, law="zipf", zipf_s=1.0, gamma=2.3, seed=31)
+    pats = random_patterns(600, range(4, 7), ALL_SHAPES, lab, 17)
+    g = fx.Graph(lab, src, dst, search_blocks=blocks)
+    w = fx.Graph(lab, src, dst, window_min=16, window_max=256)
+    mode = EARLY | fx.FLEXIS_MODE_NO_MNI
+    want = [key(r) for r in w.support_batch(pats, sigma, 0.5, mode)]
+    for _ in range(3):
+        assert [key(r) for r in g.support_batch(pats, sigma, 0.5, mode)] == want
+    g.close()
+    w.close()
