@@ -159,15 +159,18 @@ int tune_bucket(int64_t P) {
 }
 
 // Evaluate plans [lo, lo + cnt) with the autotuner's budget for the bucket (tuning it first if
-// the bucket is new).  Returns the results into out + lo.
-int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cnt, flexis_support_result *out,
-               flexis_stats &total) {
+// the bucket is new).  Returns the results into out + lo.  `streamed`: by the streaming greedy, where the
+// graph's options allow it.
+int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cnt, bool streamed,
+               flexis_support_result *out, flexis_stats &total) {
     EvalConfig c2 = config_for(g, cnt);
     enum_config(g, plans.data() + lo, cnt, c2);
+    c2.streamed &= streamed;
     const bool tunable = g->opt.autotune >= 0 && g->opt.search_budget == 0 && cnt >= TUNE_MIN && !c2.exact_mis;
     int64_t done = 0;
     if (tunable) {
-        const int bucket = tune_bucket(cnt);
+        // (what is timed under the streaming greedy says nothing about the windowed rounds)
+        const int bucket = 2 * tune_bucket(cnt) + (c2.streamed ? 1 : 0);
         auto it = g->tuned_budget.find(bucket);
         if (it == g->tuned_budget.end()) {
             // (the streaming greedy has no budget to choose: a token slice)
@@ -177,6 +180,7 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
             for (int32_t cand : TUNE_CANDIDATES) {
                 EvalConfig c3 = config_for(g, slice);
                 enum_config(g, plans.data() + lo, slice, c3);
+                c3.streamed = c2.streamed;
                 c3.search_budget = cand;
                 c3.w_min = c2.w_min;
                 c3.w_max = c2.w_max;
@@ -209,23 +213,33 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
 }
 
 // Memory-admitted batches: the device workspace of one batch (used bitmaps, windows, items) is
-// bounded by a share of the free device memory; larger candidate sets run as several batches.
+// bounded by a share of the free device memory; larger candidate sets run as several batches.  When there is no
+// room for the streaming greedy's buffers, the rest of the set is cut again for the windowed rounds.
 int eval_plans(flexis_graph *g, std::vector<Plan> &plans, flexis_support_result *out) {
     const int64_t P = (int64_t)plans.size();
     EvalConfig cfg = config_for(g, (int32_t)std::min<int64_t>(P, INT32_MAX));
     enum_config(g, plans.data(), P, cfg);
-    int64_t per = 1, fr = 0;
-    dev_pattern_bytes(g->dg, cfg.w_max, cfg.record_selected, cfg.streamed, &per);
-    dev_free_bytes(g->dg, &fr);
-    const int64_t budget = std::max<int64_t>(fr / 3, 256ll << 20);
-    int64_t chunk = std::max<int64_t>(1, std::min<int64_t>({P, budget / std::max<int64_t>(per, 1), 1 << 22}));
-    // the exact MIS materialises every map of its patterns: a few patterns at a time
-    if (cfg.exact_mis) chunk = std::min<int64_t>(chunk, EXACT_MIS_BATCH);
+    auto batch_patterns = [&] {
+        int64_t per = 1, fr = 0;
+        dev_pattern_bytes(g->dg, cfg.w_max, cfg.record_selected, cfg.streamed, &per);
+        dev_free_bytes(g->dg, &fr);
+        const int64_t budget = std::max<int64_t>(fr / 3, 256ll << 20);
+        const int64_t n = std::max<int64_t>(1, std::min<int64_t>({P, budget / std::max<int64_t>(per, 1), 1 << 22}));
+        // the exact MIS materialises every map of its patterns: a few patterns at a time
+        return cfg.exact_mis ? std::min<int64_t>(n, EXACT_MIS_BATCH) : n;
+    };
+    int64_t chunk = batch_patterns();
     flexis_stats total{};
-    for (int64_t lo = 0; lo < P; lo += chunk) {
+    for (int64_t lo = 0; lo < P;) {
         const int32_t cnt = (int32_t)std::min(chunk, P - lo);
-        int rc = eval_chunk(g, plans, lo, cnt, out, total);
+        int rc = eval_chunk(g, plans, lo, cnt, cfg.streamed, out, total);
+        if (rc == EVAL_NO_STREAM_ROOM) {
+            cfg.streamed = false;
+            chunk = batch_patterns();
+            continue;
+        }
         if (rc) return rc;
+        lo += cnt;
     }
     g->last = total;
     return FLEXIS_OK;
@@ -526,7 +540,12 @@ int flexis_support_plans_device(flexis_graph *g, const flexis_plan *d_plans, int
             return FLEXIS_E_CUDA;
         enum_config(g, h.data(), count, cfg);
     }
-    return dev_eval(g->dg, d_plans, count, d_results, s, cfg, &g->last);
+    int rc = dev_eval(g->dg, d_plans, count, d_results, s, cfg, &g->last);
+    if (rc == EVAL_NO_STREAM_ROOM) {
+        cfg.streamed = false;
+        rc = dev_eval(g->dg, d_plans, count, d_results, s, cfg, &g->last);
+    }
+    return rc;
 }
 
 int flexis_last_stats(const flexis_graph *g, flexis_stats *out) {

@@ -49,6 +49,11 @@ int64_t dev_graph_bytes(const DeviceGraph *g);
 int dev_graph_props(const DeviceGraph *g, int *sm_count, int *l2_bytes);
 cudaStream_t dev_graph_stream(const DeviceGraph *g);
 
+// Of dev_eval and dev_eval_host with cfg.streamed: no room for the streaming greedy's buffers.  Nothing has been
+// evaluated and its buffers are given back; the caller evaluates in windowed rounds, in batches cut to
+// their size (a pattern takes some hundred times the memory there).
+constexpr int EVAL_NO_STREAM_ROOM = 1;
+
 // Evaluate P compiled plans that are already in device memory; results to device memory.
 // Synchronises `stream` before returning.  stats (nullable) receives counters.
 int dev_eval(DeviceGraph *g, const flexis_plan *d_plans, int32_t P, flexis_support_result *d_results,

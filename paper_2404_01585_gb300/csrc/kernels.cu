@@ -1295,23 +1295,21 @@ static int eval_batch(DeviceGraph *g, const Plan *h_plans, const flexis_plan *ro
     const int Wmin = std::max(1, std::min(cfg.w_min, Wmax));
     if (cfg.cyclic)
         if (int rc = dev_edge_set(g)) return rc;
-    bool streamed = cfg.streamed;
+    const bool streamed = cfg.streamed;
     StreamArgs A{};
-    int rc, stream_blocks = 0;
+    int rc = FLEXIS_OK, stream_blocks = 0;
     if (streamed) {
         stream_shape(g, cfg, P, A, stream_blocks);
-        // no room for its buffers: the windowed rounds, which need less for a small batch
         rc = sws_ensure(g, A.S, (int64_t)A.S * A.RG * A.GS);
-        if (rc == FLEXIS_E_NOMEM) {
-            (void)cudaGetLastError();
-            sws_free(g->sws);
-            streamed = false;
-        } else if (rc) {
-            return rc;
-        }
     }
     const int32_t H = streamed ? 0 : P;  // the streaming greedy has bitmaps of its own and no windows
-    if ((rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected))) return rc;
+    if (!rc) rc = ws_ensure(g, g->ws, P, H, Wmax, cfg.record_selected);
+    if (rc == FLEXIS_E_NOMEM && streamed) {
+        (void)cudaGetLastError();
+        sws_free(g->sws);
+        return EVAL_NO_STREAM_ROOM;
+    }
+    if (rc) return rc;
     Workspace &w = g->ws;
     const Plan *d_plans = w.plans;
     if (h_plans) {
