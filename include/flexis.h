@@ -124,7 +124,8 @@ typedef struct {
                                 the maps committed so far (a lower bound of their mIS), mni = -1
                                 and frequent = 0 (undecided); flexis_mine then fails with
                                 FLEXIS_E_TIMEOUT.  The limit is checked between rounds of the
-                                greedy phase or every 32 chunks of a streamed search, and by the MNI kernel itself (device clock) every
+                                greedy phase, or by the streaming launch (device clock) between groups
+                                of at most 32 roots and every 32 chunks of a search, and by the MNI kernel itself (device clock) every
                                 few thousand candidate chunks of a search: a pattern whose MNI
                                 count is cut reports FLEXIS_E_TIMEOUT with its final mis and
                                 frequent and mni = -1.  0 = no limit (default). */

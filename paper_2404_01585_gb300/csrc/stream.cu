@@ -214,6 +214,18 @@ __device__ void drop_task(const Batch &B, const StreamArgs &A, int task) {
     if (atomicSub(A.block_open + b, 1) == 1) stack_push(&B.ctl->blocks_free, A.block_next, b);
 }
 
+// Whether the deadline has passed (the whole warp; lane 0 looks).  Warps look between groups, and within a long
+// search: most roots are decided in a few steps, so the searches alone would not see the clock.
+__device__ __forceinline__ bool late(const Batch &B) {
+    if (!B.deadline_ns) return false;
+    int r = 0;
+    if ((threadIdx.x & 31) == 0 && global_ns() - __ldg(&B.ctl->t0_ns) > B.deadline_ns) {
+        *reinterpret_cast<volatile int32_t *>(&B.ctl->expired) = 1;
+        r = 1;
+    }
+    return __shfl_sync(FULLMASK, r, 0) != 0;
+}
+
 // Stop rule of a stream search, every STOP_EVERY chunks: abort when the pattern is done, a task ahead
 // of this one has found a map, or the deadline has passed; cut the search when it has run for
 // `split_at` chunks and warps are idle.
@@ -885,6 +897,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
     unsigned long long key = 0;
     for (;;) {
         if (mode == M_CLAIM) {
+            if (late(B)) break;
             int nr = 0;
             if (lane == 0) nr = *reinterpret_cast<volatile int32_t *>(&B.ctl->n_ready);
             const int tk = __shfl_sync(FULLMASK, nr, 0) > 0 ? ready_take(B, A, gw) : -1;
@@ -1000,6 +1013,8 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             }
         }
         if (mode == M_RETIRE) {
+            // (a retiring warp may go on for many batches of roots that lanes search again)
+            if (res == RES_LANES && late(B)) break;
             const int rt = retire_step(G, B, A, X, s, res, root, from);
             if (rt == RT_DONE) {
                 release = true;
@@ -1087,11 +1102,6 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
             continue;
         }
         if (release) {
-            if (B.deadline_ns) {
-                bool end = false;
-                if (lane == 0) end = *reinterpret_cast<volatile int32_t *>(&B.ctl->expired);
-                if (__any_sync(FULLMASK, end)) break;
-            }
             // Whoever ends the pattern clears what this warp wrote for it (dead candidates, maps): every lane's
             // stores come before the reference falls.  An aborted search gets here with no fence of its own.
             __threadfence();

@@ -118,3 +118,31 @@ def test_slots_reused_after_aborted_searches(blocks, sigma):
         assert [key(r) for r in g.support_batch(pats, sigma, 0.5, mode)] == want
     g.close()
     w.close()
+
+
+# Roots that lanes decide in a few steps: no search is long enough to look at the clock, so the deadline has to be
+# seen between groups.  The call after it starts from buffers that the stopped one left as they were.
+@pytest.mark.parametrize("record", [0, 2])
+def test_deadline_stops_many_cheap_patterns(record):
+    lab, src, dst = er(20000, 40000, 4, 6)
+    pats = random_patterns(2000, range(3, 5), ["tree", "path"], lab, 8)
+    many = pats * 10
+    mode, sigma = EARLY | fx.FLEXIS_MODE_NO_MNI, 100_000  # never reached: every root is searched
+    ref = fx.Graph(lab, src, dst)
+    want = [key(r) for r in ref.support_batch(pats, sigma, 0.5, mode)]
+    ref.close()
+    g = fx.Graph(lab, src, dst, deadline_ms=2, record_selected=record)
+    for _ in range(2):
+        res = g.support_batch(many, sigma, 0.5, mode)
+        stopped = 0
+        for i, r in enumerate(res):
+            if r["status"] == fx.FLEXIS_E_TIMEOUT:
+                stopped += 1
+                assert 0 <= r["mis"] <= want[i % len(pats)][2] and r["mni"] == -1 and not r["frequent"]
+            else:
+                assert key(r) == want[i % len(pats)]
+        assert 0 < stopped
+        alone = [key(g.support(pl, pe, sigma, 0.5, mode=mode)) for pl, pe in pats[:8]]
+        decided = [k == w for k, w in zip(alone, want) if k[0] == 0]
+        assert decided and all(decided)
+    g.close()
