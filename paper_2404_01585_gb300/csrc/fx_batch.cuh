@@ -54,6 +54,7 @@ struct Ctl {
     int32_t expired;       // ... the deadline passed
     int32_t idlers;        // ... warps without work
     int32_t blocks_bump, teams_bump;  // ... task blocks and teams handed out for the first time
+    int32_t arrived;       // ... blocks that stay
     int32_t n_ready;       // ... tasks ready to run (about)
     unsigned long long blocks_free, teams_free;  // ... stacks of free indices (stream.cu)
     unsigned long long ready[READY_STACKS];      // ... stacks of tasks ready to run

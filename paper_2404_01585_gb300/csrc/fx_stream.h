@@ -39,6 +39,9 @@ struct StreamArgs {
     int32_t *task_next, *block_next, *block_open;  // their links; of their blocks: links, tasks open
     unsigned char *teams; // [STREAM_TEAMS][STREAM_TEAM_BYTES] shared searches
     int32_t *team_next;
+    // SMs left to other work (see k_stream): SMs from spare_sm on, the blocks that fit on them
+    int32_t spare, spare_sm;
+    int32_t keep;         // blocks below it stay to the end of the batch
 };
 
 constexpr int STREAM_GS_MIN = 4, STREAM_GS_MAX = 32;
@@ -46,6 +49,8 @@ constexpr int64_t STREAM_BITMAP_BYTES = 2ll << 30;  // used bitmaps of all slots
 constexpr int64_t STREAM_RING_ROOTS = 1 << 20;      // roots in flight over all slots, at most
 constexpr int64_t STREAM_RING_SLOT_MIN = 128, STREAM_RING_SLOT_MAX = 16384;  // ... of one slot
 constexpr int STREAM_SLOT_WARPS = 512;
+constexpr int STREAM_SPARE_DIV = 19;  // one in so many SMs is left to other work
+constexpr int STREAM_KEEP_DIV = 4;    // a quarter of a full grid stays to the end
 constexpr int STREAM_TASKS = 8192, STREAM_TASK_WORDS = 192, STREAM_TEAMS = 1024, STREAM_TEAM_BYTES = 1280;
 constexpr int64_t STREAM_MAX_ROOTS = ((1ll << 24) - 1) * STREAM_GS_MIN;  // group numbers have 24 bits
 

@@ -1258,8 +1258,10 @@ static void stream_shape(const DeviceGraph *g, const EvalConfig &cfg, int32_t P,
     constexpr int warps_per_block = SEARCH_THREADS / 32;
     const int64_t bitmap = 4ll * g->view.words;
     const int full = cfg.search_blocks > 0 ? cfg.search_blocks : g->sm_count * g->stream_per_sm;
+    const int free_sms = cfg.search_blocks > 0 ? 0 : g->sm_count / STREAM_SPARE_DIV;
+    const int spare = free_sms * g->stream_per_sm;
     // slots: one a warp when patterns are many (no map is ever stale then), never more than the warps
-    int64_t S = std::min<int64_t>({(int64_t)P, (int64_t)full * warps_per_block,
+    int64_t S = std::min<int64_t>({(int64_t)P, (int64_t)(full - spare) * warps_per_block,
                                    std::max<int64_t>(64, STREAM_BITMAP_BYTES / std::max<int64_t>(bitmap, 1))});
     S = std::max<int64_t>(1, S);
     A.S = (int32_t)S;
@@ -1271,6 +1273,9 @@ static void stream_shape(const DeviceGraph *g, const EvalConfig &cfg, int32_t P,
     A.RG = (int32_t)(rw / A.GS);
     // at most STREAM_SLOT_WARPS warps a slot: more only get in each other's way
     blocks = (int)std::min<int64_t>(full, std::max<int64_t>(1, S * STREAM_SLOT_WARPS / warps_per_block));
+    A.spare = blocks > g->sm_count - free_sms ? spare : 0;  // (fewer blocks leave SMs free anyway)
+    A.spare_sm = g->sm_count - free_sms;
+    A.keep = full / STREAM_KEEP_DIV;
     A.window0 = std::max(2, (S >= 128 ? 64 : 128) / A.GS);
 }
 
@@ -1692,9 +1697,21 @@ struct ServeSession {
     int sblocks = 0;
 };
 
+// The kernels of a serving step are loaded when the session starts: loaded at the first request instead, they
+// would wait for whatever runs on the device then.
+static int serve_load() {
+    const void *kernels[] = {(const void *)k_admit,  (const void *)k_commit<KMAP>, (const void *)k_search,
+                             (const void *)k_mni_setup, (const void *)k_mni,      (const void *)k_finalize,
+                             (const void *)k_cancel};
+    cudaFuncAttributes a;
+    for (const void *k : kernels) CK(cudaFuncGetAttributes(&a, k));
+    return FLEXIS_OK;
+}
+
 int serve_create(DeviceGraph *g, int32_t slots, int32_t wmin, int32_t wmax, int32_t budget,
                  ServeSession **out) {
     CK(cudaSetDevice(g->device));
+    if (int rc = serve_load()) return rc;
     ServeSession *s = new ServeSession();
     s->g = g;
     s->slots = slots;

@@ -65,6 +65,8 @@ constexpr int SPLIT_IDLE = 8, SPLIT_READY = 1;  // idle warps, and tasks waiting
 constexpr uint32_t SHARE_STEPS = 128;   // expected chunks of a group's open roots from which they are shared
 constexpr int STREAM_BLOCKS = 2;         // resident blocks per SM
 constexpr int STREAM_HOME = 16;         // warps that stay with a slot
+constexpr unsigned long long SPARE_WAIT = 2000000;  // ns
+constexpr int LEAVE_POLLS = 16, LEAVE_POLLS_HOME = 128;  // looks of a roaming and of a home warp in about 1 ms
 constexpr uint32_t STREAM_NAP = 1000, STREAM_NAP_HOME = 8000, STREAM_NAP_MAX = 128000;  // ns between looks
 
 // What a retiring warp keeps while one of its searches runs (the kernel has one search call, so that
@@ -867,6 +869,17 @@ __device__ __noinline__ bool cut_search(const Batch &B, const StreamArgs &A, Str
     return true;
 }
 
+// Two resident blocks take an SM's registers, and the launch lasts as long as its heaviest pattern: on all SMs it
+// would hold up every other stream of the process, servers among them, for hundreds of milliseconds.  So
+// one SM in STREAM_SPARE_DIV is left alone: a block that finds itself on one of the last SMs leaves as soon as
+// all but A.spare of the blocks run elsewhere.  (It does not leave at once: while another kernel holds the
+// other SMs, the free places would be these, and every block would pass through them.  When that kernel
+// goes on for SPARE_WAIT, it stays.)  Whole SMs, because a kernel that needs more shared memory than this one
+// left it cannot start on a shared SM.  And a block whose warps have all been idle for about a millisecond leaves, but for a quarter of the grid: what
+// becomes ready later is found by the warp that made it ready, if by no other.  Requests of a server beside
+// a batch of 4,000 on 100k vertices: p50 88 ms and p99 270 when all SMs were held, 0.8 and 1.7 now
+// (0.7 and 4.3 beside windowed rounds).  The batch takes 300 ms either way, the others timed are unchanged.
+//
 // (128 registers a thread: with 64 and twice the warps the same work took up to half as long again, the
 // kernel's spills and its misses of the instruction cache -- a third of the warps' time then -- grew.)
 template <class View>
@@ -874,10 +887,33 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                                                                          const __grid_constant__ StreamArgs A) {
     const View &G = static_cast<const View &>(B.G);
     __shared__ StreamWarp ws[STREAM_WARPS];
+    __shared__ int s_block, s_idle;  // number among the blocks that stay; warps idle for long
+    if (threadIdx.x == 0) {
+        int b = (int)blockIdx.x;
+        if (A.spare) {
+            uint32_t sm;
+            asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+            bool leave = false;
+            if ((int)sm >= A.spare_sm) {
+                const unsigned long long t0 = global_ns();
+                for (;;) {
+                    leave = *reinterpret_cast<volatile int32_t *>(&B.ctl->arrived) >= (int)gridDim.x - A.spare;
+                    if (leave || global_ns() - t0 > SPARE_WAIT) break;
+                    __nanosleep(STREAM_NAP);
+                }
+            }
+            b = leave ? -1 : atomicAdd(&B.ctl->arrived, 1);
+        }
+        s_block = b;
+        s_idle = 0;
+    }
+    __syncthreads();
+    const int block = s_block;
+    if (block < 0) return;
     const int lane = threadIdx.x & 31;
     StreamWarp &X = ws[threadIdx.x >> 5];
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    const int gw = (int)((block * blockDim.x + threadIdx.x) >> 5);
+    const int nw = (int)(((gridDim.x - A.spare) * blockDim.x) >> 5);
     if (lane == 0) X.W.acc_scanned = X.W.acc_bound = X.W.acc_maps = X.W.acc_items = 0;
     __syncwarp();
     for (int s = gw; s < A.S; s += nw) start_slot(B, A, s);
@@ -885,6 +921,7 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
     // word often; all others roam: they look over the slots at growing intervals.  (Thousands of
     // warps polling at full speed slowed every load of the searching ones several times over.)
     const int home = gw / A.S < STREAM_HOME ? gw % A.S : -1;
+    const int leave_polls = home >= 0 ? LEAVE_POLLS_HOME : LEAVE_POLLS;
     int s = gw % A.S, idle = 0, cur_p = -1;
     uint32_t nap = STREAM_NAP;
     int mode = M_CLAIM;
@@ -926,13 +963,24 @@ __global__ void __launch_bounds__(SEARCH_THREADS, STREAM_BLOCKS) k_stream(const 
                 if (g < 0) {
                     if (idle == 0 && lane == 0) atomicAdd(&B.ctl->idlers, 1);
                     if (++idle > IDLE_POLLS) break;
+                    if (block >= A.keep && idle >= leave_polls) {
+                        bool all = false;
+                        if (lane == 0) {
+                            if (idle == leave_polls) atomicAdd(&s_idle, 1);
+                            all = *reinterpret_cast<volatile int *>(&s_idle) >= STREAM_WARPS;
+                        }
+                        if (__any_sync(FULLMASK, all)) break;
+                    }
                     if (home >= 0) s = home;
                     __nanosleep(nap);
                     nap = min(nap + nap / 2, home >= 0 ? STREAM_NAP_HOME : STREAM_NAP_MAX);
                     continue;
                 }
             }
-            if (idle > 0 && lane == 0) atomicSub(&B.ctl->idlers, 1);
+            if (idle > 0 && lane == 0) {
+                atomicSub(&B.ctl->idlers, 1);
+                if (block >= A.keep && idle >= leave_polls) atomicSub(&s_idle, 1);
+            }
             nap = STREAM_NAP;
             idle = 0;
             if (tk >= 0) {

@@ -3,6 +3,9 @@ remainders, more patterns than slots, shared searches, the edge set and the coun
 quantities are integers: equality is exact."""
 from __future__ import annotations
 
+import threading
+import time
+
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -145,4 +148,41 @@ def test_deadline_stops_many_cheap_patterns(record):
         alone = [key(g.support(pl, pe, sigma, 0.5, mode=mode)) for pl, pe in pats[:8]]
         decided = [k == w for k, w in zip(alone, want) if k[0] == 0]
         assert decided and all(decided)
+    g.close()
+
+
+# A batch of some hundred milliseconds leaves SMs to other streams: requests served meanwhile are done before it,
+# also when the server is at work as the batch is launched (the last delays: after its host part of some 40 ms).
+def test_server_beside_a_batch():
+    lab, src, dst = make_graph("mico")
+    mode = EARLY | fx.FLEXIS_MODE_NO_MNI
+    big = random_patterns(6000, range(5, 7), ALL_SHAPES, lab, 7)
+    small = random_patterns(8, range(3, 5), ["tree", "path"], lab, 9)
+    g = fx.Graph(lab, src, dst)
+    want = [key(r) for r in g.support_batch(small, 300, 0.5, mode)]
+    first = [key(r) for r in g.support_batch(big, 1000, 0.5, mode)]
+    srv = fx.Server(g, slots=8)
+    for delay in (0.1, 0.08, 0.07, 0.06, 0.055, 0.05, 0.045, 0.04, 0.035, 0.03):
+        out, ended = [], threading.Event()
+
+        def batch():
+            out.extend(key(r) for r in g.support_batch(big, 1000, 0.5, mode))
+            ended.set()
+
+        t = threading.Thread(target=batch)
+        t.start()
+        time.sleep(delay)
+        for turn in range(4):
+            got = {}
+            for i, (pl, pe) in enumerate(small):
+                assert srv.submit(i, pl, pe, 300, 0.5, mode) == 0
+            while len(got) < len(small):
+                got.update((rid, r) for rid, r, _ in srv.poll())
+                time.sleep(1e-4)
+            assert [key(got[i]) for i in range(len(small))] == want
+        beside = not ended.is_set()
+        t.join()
+        assert out == first
+        assert beside, delay
+    srv.stop()
     g.close()
