@@ -801,6 +801,7 @@ struct StreamWS {
     int64_t bytes = 0;
     unsigned char *base = nullptr;  // the allocation that holds the buffers
     bool clean = false;
+    size_t zero_bytes = 0;  // from `words` on: claim and status words, bitmaps, dead candidates
     unsigned long long *words = nullptr;
     void *slots = nullptr;
     uint32_t *status = nullptr, *mask = nullptr, *used = nullptr, *dead = nullptr;
@@ -830,6 +831,7 @@ struct DeviceGraph {
     cudaGraphExec_t round_exec = nullptr;  // the captured round loop of the last level
     cudaGraphExec_t stream_exec = nullptr; // the captured streaming evaluation,
     std::vector<unsigned char> stream_key; // what it was launched with,
+    std::vector<unsigned char> stream_seen; // what the call before was launched with
     int64_t stream_nodes = 0;              // its kernels
     std::vector<cudaEvent_t> gev;          // search-launch events of a group of rounds
     int64_t graph_instantiations = 0, graph_fallbacks = 0;

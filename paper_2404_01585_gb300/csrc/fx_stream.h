@@ -55,8 +55,9 @@ constexpr int STREAM_TASKS = 8192, STREAM_TASK_WORDS = 192, STREAM_TEAMS = 1024,
 constexpr int64_t STREAM_MAX_ROOTS = ((1ll << 24) - 1) * STREAM_GS_MIN;  // group numbers have 24 bits
 
 int stream_blocks_per_sm();
-// `cyclic`: some pattern has a cycle.
-void launch_stream(const Batch &B, const StreamArgs &A, bool cyclic, int blocks, cudaStream_t stream);
+// Whether the kernel for graphs with all their tables runs; `cyclic`: some pattern has a cycle.
+inline bool stream_fast(const Batch &B, bool cyclic) { return B.G.off && (B.G.edges || !cyclic) && !B.sel; }
+void launch_stream(const Batch &B, const StreamArgs &A, bool fast, int blocks, cudaStream_t stream);
 // After the stream kernel: when the deadline passed, the patterns it left undecided.
 void launch_stream_expire(const Batch &B, const StreamArgs &A, cudaStream_t stream);
 

@@ -1377,8 +1377,8 @@ int stream_blocks_per_sm() {
     return per_sm < 1 ? 1 : per_sm;
 }
 
-void launch_stream(const Batch &B, const StreamArgs &A, bool cyclic, int blocks, cudaStream_t stream) {
-    if (B.G.off && (B.G.edges || !cyclic) && !B.sel)
+void launch_stream(const Batch &B, const StreamArgs &A, bool fast, int blocks, cudaStream_t stream) {
+    if (fast)
         k_stream<FastView><<<blocks, SEARCH_THREADS, 0, stream>>>(B, A);
     else
         k_stream<DevGraphView><<<blocks, SEARCH_THREADS, 0, stream>>>(B, A);

@@ -186,3 +186,28 @@ def test_server_beside_a_batch():
         assert beside, delay
     srv.stop()
     g.close()
+
+
+# A call of a few patterns is captured when it comes a second time; calls of two kinds in turn are launched singly.
+def test_small_calls_are_captured_on_their_second_launch():
+    lab, src, dst = er(3000, 12000, 4, 5)
+    g = fx.Graph(lab, src, dst)
+    tree = (np.array([0, 1, 2], np.int32), np.array([[0, 1], [1, 2]], np.int32))
+    ring = (np.array([0, 1, 2], np.int32), np.array([[0, 1], [1, 2], [2, 0]], np.int32))
+    w = fx.Graph(lab, src, dst, window_min=16, window_max=256)
+
+    def replays(calls):
+        out = []
+        for (pl, pe), mode in calls:
+            assert key(g.support(pl, pe, 50, 0.5, mode=mode)) == key(w.support(pl, pe, 50, 0.5, mode=mode))
+            out.append(g.stats()["graph_launches"])
+        return out
+
+    plain = EARLY | fx.FLEXIS_MODE_NO_MNI
+    assert replays([(tree, FULL)] * 3) == [0, 1, 1]
+    # the edge set is built for the first cycle; from then on trees and cycles are one kind
+    assert replays([(ring, FULL), (tree, FULL), (ring, FULL)]) == [0, 1, 1]
+    assert replays([(tree, plain), (tree, FULL), (ring, plain), (ring, FULL)]) == [0, 1, 0, 1]
+    assert replays([(tree, plain), (ring, plain), (tree, FULL), (tree, plain)]) == [0, 1, 0, 1]
+    g.close()
+    w.close()
