@@ -105,11 +105,11 @@ EvalConfig config_for(const flexis_graph *g, int32_t P) {
     int wmin = std::max(16, std::min(wmax, 16384 / std::max(1, P)));
     if (g->opt.window_max > 0) wmax = g->opt.window_max;
     if (g->opt.window_min > 0) wmin = g->opt.window_min;
-    // the streaming greedy, unless the caller sets up the windowed rounds himself (or a label may
-    // have more roots than it can number)
+    // the streaming greedy, unless the caller sets up the windowed rounds (or a label may have more
+    // roots than it can number)
     const flexis_options &o = g->opt;
     c.streamed = o.window_max <= 0 && o.window_min <= 0 && o.search_budget == 0 && o.split_pieces == 0 &&
-                 o.sub_searches <= 0 && g->hg.nv < (int64_t)60'000'000;
+                 o.sub_searches <= 0 && g->hg.nv < STREAM_MAX_VERTICES;
     c.w_min = std::min(wmin, wmax);
     c.w_max = wmax;
     c.search_blocks = g->opt.search_blocks;

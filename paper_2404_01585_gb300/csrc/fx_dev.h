@@ -6,6 +6,10 @@
 
 namespace fx {
 
+// The streaming greedy numbers the groups of a pattern's roots in 24 bits and keeps vertex + 1 in 27 (stream.cu,
+// fx_kern.cuh); from so many vertices on the windowed rounds run.
+constexpr int64_t STREAM_MAX_VERTICES = 60'000'000;
+
 struct DeviceGraph;  // resident CSR + label index + per-graph evaluation workspace
 
 struct EvalConfig {

@@ -419,7 +419,7 @@ struct BudgetStop {
 // chunk of level i is tested, every lane also fetches the slice that its candidate gives level
 // i + 1; binding a candidate then needs no look-up.  The last level is not entered candidate by
 // candidate: all (candidate of level n-2, entry of its slice) pairs of a chunk are tested 32 at a
-// time, in lexicographic order (`expand` below).  Together with the slice table and the four-way
+// time, in lexicographic order (`expand` below).  Together with the slice table and the eight-way
 // membership search this took the level-4 candidates of that run from 6.4 M entered levels and as
 // many chunks, one after another, to 3.1 M chunks and 1.1 M pair rounds.
 // ROOT_KNOWN: the caller has tested the root and passes its level-1 slice.  dead (nullable): the

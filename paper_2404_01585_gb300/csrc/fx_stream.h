@@ -52,7 +52,6 @@ constexpr int STREAM_SLOT_WARPS = 512;
 constexpr int STREAM_SPARE_DIV = 19;  // one in so many SMs is left to other work
 constexpr int STREAM_KEEP_DIV = 4;    // a quarter of a full grid stays to the end
 constexpr int STREAM_TASKS = 8192, STREAM_TASK_WORDS = 192, STREAM_TEAMS = 1024, STREAM_TEAM_BYTES = 1280;
-constexpr int64_t STREAM_MAX_ROOTS = ((1ll << 24) - 1) * STREAM_GS_MIN;  // group numbers have 24 bits
 
 int stream_blocks_per_sm();
 // Whether the kernel for graphs with all their tables runs; `cyclic`: some pattern has a cycle.

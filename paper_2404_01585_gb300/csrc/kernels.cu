@@ -125,7 +125,7 @@ __device__ __forceinline__ void save_state(uint32_t *dst, const WarpState &W, in
 // One warp per work item.  Item (pattern, slot): a fresh search for the first map of the slot's
 // root avoiding the used set.  Item (pattern, slot, saved sub-search): continue that sub-search.
 // A search that uses up its per-round budget is saved; if it heads its slot it is also split:
-// the unscanned candidates of its shallowest level with any left go to up to five new
+// the unscanned candidates of its shallowest level with any left go to up to fifteen new
 // sub-searches, in order, and a continuation takes over everything after them.  Once all but an
 // eighth of the launch's warps have found the item list empty, the searches still running are
 // saved (and split) the same way at their next drain check instead of running to the budget,
@@ -159,12 +159,11 @@ __global__ void __launch_bounds__(SEARCH_THREADS, 4) k_search(Batch B, int q) {
         const int off = item.y & 0xFFFFFF;
         const int sid_in = (item.y >> 24) - 1;
         const Plan &P = B.plans[p];
-        const size_t h = (size_t)p;
-        const size_t slot = h * 2 * B.Wmax + off;
+        const size_t slot = (size_t)p * 2 * B.Wmax + off;
         int32_t *seq = B.win_map + slot * MAXN;
         const int32_t root = B.win_root[slot];
-        const uint32_t *used = B.used + h * B.G.words;
-        uint32_t *sbase = B.susp + h * KSUSP * DFS_SAVE_STRIDE;
+        const uint32_t *used = B.used + (size_t)p * B.G.words;
+        uint32_t *sbase = B.susp + (size_t)p * KSUSP * DFS_SAVE_STRIDE;
         const bool resume = sid_in >= 0;
         load_level_plan(W, P.greedy, P);
         if (resume) {
@@ -325,13 +324,12 @@ __device__ __forceinline__ void commit_one(const Batch &B, int q, int p, int32_t
     const int nwin = S->nwin;
     const int Wmax = B.Wmax;
     const int cur = S->buf, nxt = cur ^ 1;
-    const size_t h = (size_t)p;
-    const size_t pb = h * 2 * Wmax;
+    const size_t pb = (size_t)p * 2 * Wmax;
     const size_t cb = pb + (size_t)cur * Wmax, nb = pb + (size_t)nxt * Wmax;
     const int32_t *st_cur = B.win_state + cb, *rt_cur = B.win_root + cb, *mp_cur = B.win_map + cb * MAXN;
     int32_t *st_nxt = B.win_state + nb, *rt_nxt = B.win_root + nb, *mp_nxt = B.win_map + nb * MAXN;
-    uint32_t *used = B.used + h * B.G.words;
-    uint32_t *sbase = B.susp + h * KSUSP * DFS_SAVE_STRIDE;
+    uint32_t *used = B.used + (size_t)p * B.G.words;
+    uint32_t *sbase = B.susp + (size_t)p * KSUSP * DFS_SAVE_STRIDE;
 
     // 0. sub-search sequences: drop sub-searches that found nothing; a slot whose first
     //    remaining sub-search found a map takes that map (if a vertex of it has been used since,
@@ -456,7 +454,7 @@ __device__ __forceinline__ void commit_one(const Batch &B, int q, int p, int32_t
                 const uint32_t old = atomicOr(used + wi, 1u << (m[l] & 31));
                 if (old == 0 && B.dirty) {  // first bit of this word: list it for the clean-up
                     const int k = atomicAdd(&S->ndirty, 1);
-                    if (k < DIRTY_CAP) B.dirty[h * DIRTY_CAP + k] = (int32_t)wi;
+                    if (k < DIRTY_CAP) B.dirty[(size_t)p * DIRTY_CAP + k] = (int32_t)wi;
                 }
             }
             const int64_t at = count0 + ncommit + excl;

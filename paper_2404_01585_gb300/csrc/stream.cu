@@ -47,6 +47,8 @@ namespace {
 constexpr int STREAM_WARPS = SEARCH_THREADS / 32;
 constexpr unsigned long long W_FIELD = (1ull << 24) - 1;
 constexpr int W_NEXT = 24, W_REFS = 48;
+static_assert(STREAM_MAX_VERTICES <= (int64_t)W_FIELD * STREAM_GS_MIN, "group numbers");
+static_assert(STREAM_MAX_VERTICES < 1ll << 27, "keys of dead candidates");
 constexpr unsigned long long W_REF1 = 1ull << W_REFS, W_REFMASK = (1ull << 14) - 1;
 constexpr unsigned long long W_ACTIVE = 1ull << 62, W_DONE = 1ull << 63;
 enum : uint32_t { G_DONE = 1u, G_HEAD = 2u };
