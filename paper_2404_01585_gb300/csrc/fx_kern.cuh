@@ -727,20 +727,21 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     return v;
 }
 
-// Block-wide exclusive scan of one int per thread; returns the total.
-__device__ __forceinline__ int block_scan(int v, int &excl, int *sh /* >= 33 ints */) {
+// Block-wide exclusive scan of one number per thread; returns the total.
+template <class T>
+__device__ __forceinline__ T block_scan(T v, T &excl, T *sh /* >= 33 entries */) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int x = v;
+    T x = v;
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULLMASK, x, o);
+        const T y = __shfl_up_sync(FULLMASK, x, o);
         if (lane >= o) x += y;
     }
     if (lane == 31) sh[w] = x;
     __syncthreads();
     if (w == 0) {
-        int t = lane < nw ? sh[lane] : 0;
+        T t = lane < nw ? sh[lane] : 0;
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(FULLMASK, t, o);
+            const T y = __shfl_up_sync(FULLMASK, t, o);
             if (lane >= o) t += y;
         }
         if (lane < nw) sh[lane] = t;  // inclusive prefix of warp totals
@@ -748,7 +749,7 @@ __device__ __forceinline__ int block_scan(int v, int &excl, int *sh /* >= 33 int
     }
     __syncthreads();
     excl = x - v + (w > 0 ? sh[w - 1] : 0);
-    const int total = sh[32];
+    const T total = sh[32];
     __syncthreads();
     return total;
 }

@@ -619,8 +619,9 @@ __global__ void __launch_bounds__(COMMIT_THREADS) k_commit(Batch B, int q) {
 
 // MNI segments: for every pattern whose mIS stayed below c and is not zero, one segment per
 // orbit covering the orbit label's vertices.
+// (Sums in 64 bits: a thousand segments of two million vertices pass 2^31.)
 __global__ void k_mni_setup(Batch B) {
-    __shared__ int sh[40];
+    __shared__ unsigned long long sh[40];
     __shared__ unsigned long long carry;
     const int tid = threadIdx.x;
     const int nseg = B.P * MAXN;
@@ -628,7 +629,7 @@ __global__ void k_mni_setup(Batch B) {
     __syncthreads();
     for (int base = 0; base < nseg; base += blockDim.x) {
         const int sidx = base + tid;
-        int len = 0;
+        unsigned long long len = 0;
         if (sidx < nseg) {
             const int p = sidx / MAXN, o = sidx % MAXN;
             const Plan &P = B.plans[p];
@@ -639,14 +640,14 @@ __global__ void k_mni_setup(Batch B) {
                               (P.skip_mis || (S.count < P.cap && S.count > 0));
             if (need && o < P.n_orb) {
                 const int u = P.orb[o].vert[0];
-                len = P.lab_end[u] - P.lab_begin[u];
+                len = (unsigned long long)(P.lab_end[u] - P.lab_begin[u]);
             }
         }
-        int excl;
-        const int tot = block_scan(len, excl, sh);
-        if (sidx < nseg) B.mni_seg[sidx] = carry + (unsigned long long)excl;
+        unsigned long long excl;
+        const unsigned long long tot = block_scan(len, excl, sh);
+        if (sidx < nseg) B.mni_seg[sidx] = carry + excl;
         __syncthreads();
-        if (tid == 0) carry += (unsigned long long)tot;
+        if (tid == 0) carry += tot;
         __syncthreads();
     }
     if (tid == 0) {
