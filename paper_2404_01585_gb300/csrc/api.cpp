@@ -150,7 +150,7 @@ void enum_config(const flexis_graph *g, const Plan *plans, int64_t n, EvalConfig
 // (device time) is kept for the graph and used for the rest of that batch and every later batch
 // of the bucket.  All budgets give the same results, so the slice's results are kept as well.
 constexpr int32_t TUNE_MIN = 4096;
-constexpr int32_t TUNE_CANDIDATES[3] = {1024, 4096, 16384};
+constexpr int32_t TUNE_CANDIDATES[3] = {1024, 4096, 16384}, TUNE_DEFAULT = 4096;
 
 int tune_bucket(int64_t P) {
     int b = 0;
@@ -173,7 +173,7 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
         const int bucket = 2 * tune_bucket(cnt) + (c2.streamed ? 1 : 0);
         auto it = g->tuned_budget.find(bucket);
         if (it == g->tuned_budget.end()) {
-            // (the streaming greedy has no budget to choose: a token slice)
+            // (the streaming greedy has no budget to choose: a token slice, and the default is reported)
             const int32_t slice = c2.streamed ? 32 : std::max<int32_t>(512, std::min<int32_t>(cnt / 8, 8192));
             float best_ms = 0.f;
             int32_t best = 0;
@@ -195,6 +195,7 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
                     best = cand;
                 }
             }
+            if (c2.streamed) best = TUNE_DEFAULT;
             it = g->tuned_budget.emplace(bucket, best).first;
             done = slice;  // every candidate gave these results
         }
@@ -206,7 +207,7 @@ int eval_chunk(flexis_graph *g, std::vector<Plan> &plans, int64_t lo, int32_t cn
         if (rc) return rc;
         st.patterns = cnt - done;
         st.batches = 1;
-        st.search_budget = c2.search_budget ? c2.search_budget : 4096;
+        st.search_budget = c2.search_budget ? c2.search_budget : TUNE_DEFAULT;
         add_stats(total, st);
     }
     return FLEXIS_OK;

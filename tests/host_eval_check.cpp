@@ -2,6 +2,7 @@
 // is cut into batches when the streaming greedy's buffers find no room.  The stand-in holds FREE bytes, takes
 // STREAM bytes for the streaming buffers and WINDOWED a pattern for the windowed rounds, and refuses what
 // does not fit.
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -42,6 +43,7 @@ static int fake_eval(const Plan *plans, int32_t P, flexis_support_result *out, c
         return FLEXIS_E_NOMEM;
     }
     calls.push_back({cfg.streamed, P});
+    if (st) st->total_ms = cfg.search_budget > 0 ? 1e6f / (float)cfg.search_budget : 1e6f;  // the largest budget is fastest
     for (int32_t i = 0; i < P && out; i++) {
         memset(&out[i], 0, sizeof out[i]);
         out[i].status = plans[i].status;
@@ -180,6 +182,36 @@ int main() {
             CHECK(res[(size_t)i].sigma == i + 1 && res[(size_t)i].rounds == (i < first ? 1 : 2));
         CHECK(calls.size() > 1 && calls[0].streamed && calls[0].P == first);
         for (size_t k = 1; k < calls.size(); k++) CHECK(!calls[k].streamed);
+        flexis_free_graph(g);
+    }
+    // a budget timed under the streaming greedy, which has none, is not the windowed rounds': those time their own
+    {
+        flexis_options opt;
+        flexis_default_options(&opt);
+        flexis_graph *g = nullptr;
+        free_bytes = 4ll << 30;
+        stream_bytes = 0;
+        streamed_room = 0;
+        CHECK(flexis_load_graph(4, labels, 3, src, dst, &opt, &g) == FLEXIS_OK);
+        const int32_t count = 6000;
+        flexis_pattern p;
+        memset(&p, 0, sizeof p);
+        p.n = 2;
+        p.m = 1;
+        p.labels = pl;
+        p.edges = pe;
+        std::vector<flexis_pattern> pats((size_t)count, p);
+        std::vector<int64_t> sigma((size_t)count, 3);
+        std::vector<double> lam((size_t)count, 0.5);
+        std::vector<flexis_support_result> res((size_t)count);
+        for (int turn = 0; turn < 3; turn++) {
+            if (turn == 1) stream_bytes = free_bytes + 1;
+            CHECK(flexis_support_batch(g, pats.data(), sigma.data(), lam.data(), count, FLEXIS_MODE_EARLY, res.data()) == FLEXIS_OK);
+            flexis_stats st;
+            CHECK(flexis_last_stats(g, &st) == FLEXIS_OK);
+            CHECK(st.autotune_probes == (turn < 2 ? 3 : 0));
+            CHECK(st.search_budget == (turn == 0 ? 4096 : 16384));
+        }
         flexis_free_graph(g);
     }
     printf("fails %d\n", fails);
