@@ -211,3 +211,26 @@ def test_small_calls_are_captured_on_their_second_launch():
     assert replays([(tree, plain), (ring, plain), (tree, FULL), (tree, plain)]) == [0, 1, 0, 1]
     g.close()
     w.close()
+
+
+# Two graphs evaluated at once from two threads: the second launch finds only the SMs that the first has left alone.
+def test_two_batches_at_once():
+    mode = EARLY | fx.FLEXIS_MODE_NO_MNI
+    lab, src, dst = make_graph("mico")
+    pats = [random_patterns(n, range(4, 7), ALL_SHAPES, lab, s) for n, s in ((3000, 7), (700, 8))]
+    gs = [fx.Graph(lab, src, dst) for _ in pats]
+    want = [[key(r) for r in g.support_batch(p, 1000, 0.5, mode)] for g, p in zip(gs, pats)]
+    for _ in range(3):
+        out = [None, None]
+
+        def batch(i):
+            out[i] = [key(r) for r in gs[i].support_batch(pats[i], 1000, 0.5, mode)]
+
+        ts = [threading.Thread(target=batch, args=(i,)) for i in (0, 1)]
+        for t in ts:
+            t.start()
+        for t in ts:
+            t.join()
+        assert out == want
+    for g in gs:
+        g.close()
