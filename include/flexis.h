@@ -17,7 +17,10 @@
  *     library copies what it keeps).  Handles (flexis_graph, flexis_pattern_set, flexis_server)
  *     are owned by the library and released with the matching flexis_free_* / _stop call.
  *   - Threading: a flexis_graph is thread-compatible, not thread-safe: calls on one handle must
- *     not overlap.  Different handles are independent.  A server owns its own host thread.
+ *     not overlap.  Different handles are independent.  A server owns its own host thread; calls on
+ *     its graph may run beside it.  One evaluation is one launch that can last seconds: it leaves one
+ *     SM in 76 to other streams, one in 8 while its graph has a server, and gives back SMs that run
+ *     out of work.
  *   - Pointers are host pointers unless the parameter name starts with `d_` (device pointer on
  *     the graph's GPU).
  *   - Exactness: every count is an integer computed exactly; results do not depend on batch
@@ -120,13 +123,13 @@ typedef struct {
     int32_t deadline_ms;     /* > 0: wall-clock limit of one evaluation call (support, batch, each
                                 device batch of a mining level) and of one served request (from
                                 its submission).  Patterns still undecided when it passes stop
-                                (between two rounds, or within a search) and report status FLEXIS_E_TIMEOUT, with mis =
-                                the maps committed so far (a lower bound of their mIS), mni = -1
+                                (between two rounds or groups of roots, or within a search) and
+                                report status FLEXIS_E_TIMEOUT, with mis = the maps committed so far (a lower bound of their mIS), mni = -1
                                 and frequent = 0 (undecided); flexis_mine then fails with
                                 FLEXIS_E_TIMEOUT.  The limit is checked between rounds of the
                                 greedy phase, or by the streaming launch (device clock) between groups
-                                of at most 32 roots and every 32 chunks of a search, and by the MNI kernel itself (device clock) every
-                                few thousand candidate chunks of a search: a pattern whose MNI
+                                of at most 32 roots and every 32 chunks of a search, and by the MNI
+                                kernel itself (device clock) every few thousand candidate chunks of a search: a pattern whose MNI
                                 count is cut reports FLEXIS_E_TIMEOUT with its final mis and
                                 frequent and mni = -1.  0 = no limit (default). */
     int32_t root_order;      /* greedy root order (Sec. 3.2.2): 0 = by (H(seed, v), v), the seeded
@@ -431,8 +434,8 @@ int64_t flexis_generate_candidates(const flexis_pattern *frequent, int32_t count
  * being evaluated, and share the device rounds with them.  A slot (used-vertex bitmap, window,
  * state: the device memory one request holds) is the admission unit; slots <= 0 sizes the
  * server from a quarter of the free device memory.  The server's host thread runs rounds of 256
- * candidate chunks per search and request on its own CUDA stream.  The graph's options.deadline_ms, when set, bounds each request from its
- * submission: a request past it is reported with status FLEXIS_E_TIMEOUT (see flexis_options).
+ * candidate chunks per search and request on its own CUDA stream.  The graph's options.deadline_ms,
+ * when set, bounds each request from its submission: a request past it is reported with status FLEXIS_E_TIMEOUT (see flexis_options).
  * window_min / window_max / search_budget of the graph's options, when set, replace the
  * server's own defaults (start window 32, at most 2048).                                      */
 int flexis_serve_start(flexis_graph *g, int32_t slots, flexis_server **out);

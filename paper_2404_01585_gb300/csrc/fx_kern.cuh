@@ -5,6 +5,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <chrono>
 #include <cstdio>
 #include <vector>
@@ -826,6 +827,7 @@ struct DeviceGraph {
     Workspace ws;
     StreamWS sws;
     int stream_per_sm = 0;  // resident blocks of the streaming kernel per SM
+    std::atomic<int32_t> servers{0};  // live serving sessions
     int32_t last_P = 0, last_sel = 0;
     cudaEvent_t ev[2]{};
     std::vector<cudaEvent_t> sev;

@@ -49,7 +49,7 @@ constexpr int64_t STREAM_BITMAP_BYTES = 2ll << 30;  // used bitmaps of all slots
 constexpr int64_t STREAM_RING_ROOTS = 1 << 20;      // roots in flight over all slots, at most
 constexpr int64_t STREAM_RING_SLOT_MIN = 128, STREAM_RING_SLOT_MAX = 16384;  // ... of one slot
 constexpr int STREAM_SLOT_WARPS = 512;
-constexpr int STREAM_SPARE_DIV = 19;  // one in so many SMs is left to other work
+constexpr int STREAM_SPARE_DIV = 76, STREAM_SPARE_DIV_SERVED = 8;  // one in so many SMs is left to other work
 constexpr int STREAM_KEEP_DIV = 4;    // a quarter of a full grid stays to the end
 constexpr int STREAM_TASKS = 8192, STREAM_TASK_WORDS = 192, STREAM_TEAMS = 1024, STREAM_TEAM_BYTES = 1280;
 

@@ -1258,7 +1258,7 @@ static void stream_shape(const DeviceGraph *g, const EvalConfig &cfg, int32_t P,
     constexpr int warps_per_block = SEARCH_THREADS / 32;
     const int64_t bitmap = 4ll * g->view.words;
     const int full = cfg.search_blocks > 0 ? cfg.search_blocks : g->sm_count * g->stream_per_sm;
-    const int free_sms = cfg.search_blocks > 0 ? 0 : g->sm_count / STREAM_SPARE_DIV;
+    const int free_sms = cfg.search_blocks > 0 ? 0 : g->sm_count / (g->servers > 0 ? STREAM_SPARE_DIV_SERVED : STREAM_SPARE_DIV);
     const int spare = free_sms * g->stream_per_sm;
     // slots: one a warp when patterns are many (no map is ever stale then), never more than the warps
     int64_t S = std::min<int64_t>({(int64_t)P, (int64_t)(full - spare) * warps_per_block,
@@ -1699,6 +1699,7 @@ struct ServeSession {
     flexis_support_result *h_res = nullptr;  // pinned
     int64_t round = 0;
     int sblocks = 0;
+    bool counted = false;  // in the graph's count of sessions
 };
 
 // The kernels of a serving step are loaded when the session starts: loaded at the first request instead, they
@@ -1745,6 +1746,8 @@ int serve_create(DeviceGraph *g, int32_t slots, int32_t wmin, int32_t wmax, int3
     Batch B = make_batch(g, s->w, s->w.plans, slots, s->Wmin, s->Wmax, 0, s->w.results);
     k_reset_ctl<<<1, 1, 0, s->stream>>>(B);
     CK(cudaStreamSynchronize(s->stream));
+    s->counted = true;
+    g->servers++;
     *out = s;
     return FLEXIS_OK;
 }
@@ -1753,6 +1756,7 @@ void serve_destroy(ServeSession *s) {
     if (!s) return;
     cudaSetDevice(s->g->device);
     if (s->stream) cudaStreamSynchronize(s->stream);
+    if (s->counted) s->g->servers--;
     ws_free(s->w);
     cudaFree(s->d_admit);
     if (s->h_admit) cudaFreeHost(s->h_admit);

@@ -873,14 +873,18 @@ __device__ __noinline__ bool cut_search(const Batch &B, const StreamArgs &A, Str
 
 // Two resident blocks take an SM's registers, and the launch lasts as long as its heaviest pattern: on all SMs it
 // would hold up every other stream of the process, servers among them, for hundreds of milliseconds.  So
-// one SM in STREAM_SPARE_DIV is left alone: a block that finds itself on one of the last SMs leaves as soon as
-// all but A.spare of the blocks run elsewhere.  (It does not leave at once: while another kernel holds the
+// one SM in 76 is left alone, one in 8 while the graph has a server: a block that finds itself on one of the
+// last SMs leaves as soon as all but A.spare of the blocks run elsewhere.  (It does not leave at once: while another kernel holds the
 // other SMs, the free places would be these, and every block would pass through them.  When that kernel
 // goes on for SPARE_WAIT, it stays.)  Whole SMs, because a kernel that needs more shared memory than this one
 // left it cannot start on a shared SM.  And a block whose warps have all been idle for about a millisecond leaves, but for a quarter of the grid: what
-// becomes ready later is found by the warp that made it ready, if by no other.  Requests of a server beside
-// a batch of 4,000 on 100k vertices: p50 88 ms and p99 270 when all SMs were held, 0.8 and 1.7 now
-// (0.7 and 4.3 beside windowed rounds).  The batch takes 300 ms either way, the others timed are unchanged.
+// becomes ready later is found by the warp that made it ready, if by no other.
+//
+// Requests of a server on another graph beside a batch of 4,000 on 100k vertices: p50 88 ms and p99 270 when
+// all SMs were held, 0.8 and 2.8 with 2 of 152 SMs free (0.7 and 4.3 beside windowed rounds).  Blocks that
+// leave cost nothing; deep mining, which fills the chip, takes 0.7 % longer with 2 SMs free, 1.8 % with 4
+// and 2.7 % with 8.  A stream of heavy requests, though, ends at 71 ms with 8 SMs, 83 with 4 and 90
+// with 2 (77 beside windowed rounds), hence the more SMs for a graph that is being served.
 //
 // (128 registers a thread: with 64 and twice the warps the same work took up to half as long again, the
 // kernel's spills and its misses of the instruction cache -- a third of the warps' time then -- grew.)
