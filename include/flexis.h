@@ -119,18 +119,19 @@ typedef struct {
     int32_t sub_searches;    /* saved sub-searches a pattern may hold at once (1..32): 0 = default */
     int32_t timing;          /* 1: CUDA events around every search launch (stats.search_ms) */
     int32_t graphs;          /* 0 = default (an evaluation's launches, or its round loop, are captured
-                                into a CUDA graph and replayed), -1 = launch kernel by kernel */
+                                into a CUDA graph and replayed; fewer than 32 patterns when the
+                                same call comes again), -1 = launch kernel by kernel */
     int32_t deadline_ms;     /* > 0: wall-clock limit of one evaluation call (support, batch, each
                                 device batch of a mining level) and of one served request (from
                                 its submission).  Patterns still undecided when it passes stop
                                 (between two rounds or groups of roots, or within a search) and
-                                report status FLEXIS_E_TIMEOUT, with mis = the maps committed so far (a lower bound of their mIS), mni = -1
-                                and frequent = 0 (undecided); flexis_mine then fails with
-                                FLEXIS_E_TIMEOUT.  The limit is checked between rounds of the
+                                report status FLEXIS_E_TIMEOUT, with mis = the maps committed so far
+                                (a lower bound of their mIS), mni = -1 and frequent = 0 (undecided);
+                                flexis_mine then fails with FLEXIS_E_TIMEOUT.  The limit is checked between rounds of the
                                 greedy phase, or by the streaming launch (device clock) between groups
                                 of at most 32 roots and every 32 chunks of a search, and by the MNI
-                                kernel itself (device clock) every few thousand candidate chunks of a search: a pattern whose MNI
-                                count is cut reports FLEXIS_E_TIMEOUT with its final mis and
+                                kernel itself (device clock) every few thousand candidate chunks of
+                                a search: a pattern whose MNI count is cut reports FLEXIS_E_TIMEOUT with its final mis and
                                 frequent and mni = -1.  0 = no limit (default). */
     int32_t root_order;      /* greedy root order (Sec. 3.2.2): 0 = by (H(seed, v), v), the seeded
                                 hash order (default); 1 = by vertex id, the order in which the
